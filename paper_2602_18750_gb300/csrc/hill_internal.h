@@ -100,6 +100,7 @@ struct QuantArgs {
   int64_t k_sb, k_sh, k_sn;
   uint8_t* k8;                // [B][Hkv][cap][128] E4M3 codes
   float* kscale;              // [B][Hkv][cap32]
+  int chunks;                 // chunks of rows per (b, g), one warp each (set by the launcher)
 };
 
 struct SelectArgs {

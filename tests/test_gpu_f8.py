@@ -68,6 +68,41 @@ def test_quantize_k_bit_exact(H, oracle_mod, dtype):
         assert np.all(got_s[b, :, : begin[b]] == -1.0)
 
 
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("pad", [0, 8, 16])
+@pytest.mark.parametrize("rows", [1, 3, 4, 5, 15, 16, 17, 33])
+def test_quantize_k_row_counts(H, oracle_mod, rows, pad, dtype):
+    """Row counts at the edges of a warp's 16 rows, rows that start on 32 bytes and rows that start on 16 only,
+    subnormal values: exactly the requested rows are written, bit for bit, also where the sequences ask for different
+    counts under one max_rows."""
+    B, Hkv, cap = 3, 3, 60
+    g = torch.Generator().manual_seed(rows)
+    K = torch.randn(B, Hkv, cap, 128, generator=g)
+    # rows of subnormals in fp16; in bf16 as small as a row may be: 448 / amax has to be finite in float32, so
+    # amax > 448 / 3.4e38 = 1.3e-36 (below it the oracle and the kernel treat the zeros of a row differently)
+    K[0, 2] *= 1e-6 if dtype == torch.float16 else 1e-35
+    K = K.to(dtype)
+    K[0, 1, 5] = 0
+    Kd = torch.zeros(B, Hkv, cap, 128 + pad, dtype=dtype, device="cuda")[..., pad:]
+    Kd.copy_(K)
+    desc = H.make_desc(torch.zeros(B, Hkv, 128, dtype=dtype, device="cuda"), Kd)
+    k8, ks = H.alloc_shadow(desc)
+    k8.fill_(0xAB)
+    ks.fill_(-1.0)
+    begin = [5, cap - rows, 0]
+    end = [5 + rows, cap, rows // 2]
+    H.hill_quantize_k(desc, Kd, _i32(begin), _i32(end), rows, k8, ks)
+    H.hill_sync_status()
+    codes, scale = oracle_mod.quantize_rows(K)
+    got_c, got_s = k8.cpu().numpy(), ks.cpu().numpy()
+    for b in range(B):
+        inside = np.zeros(cap, dtype=bool)
+        inside[begin[b]:end[b]] = True
+        assert np.array_equal(got_c[b][:, inside], codes[b][:, inside])
+        assert np.array_equal(got_s[b, :, :cap][:, inside], scale[b][:, inside])
+        assert np.all(got_c[b][:, ~inside] == 0xAB) and np.all(got_s[b, :, :cap][:, ~inside] == -1.0)
+
+
 def test_quantize_k_token_major_layout(H, oracle_mod):
     """A token-major cache [B][cap][Hkv][d] quantises to the same dense shadow."""
     B, Hkv, cap = 2, 2, 97
