@@ -186,8 +186,7 @@ hill_status check_desc(const hill_desc* d) {
   // passes (head_passes)
   if (d->batch > score_max_batch() || d->batch > attn_max_batch()) return HILL_ERR_UNSUPPORTED;
   // the selection keeps a sequence's keys on chip across at most 8 CTAs
-  if (select_smem_bytes(d->capacity, select_cluster_size(d->capacity)) > 220 * 1024)
-    return HILL_ERR_UNSUPPORTED;
+  if (!select_cap_ok(d->capacity)) return HILL_ERR_UNSUPPORTED;
   return HILL_OK;
 }
 
@@ -444,7 +443,7 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
 hill_status run_select(const hill_desc* d, const float* key, const int32_t* lens, const int32_t* k,
                        int max_k, int32_t* idx, int32_t* count, const DeviceInfo& di, cudaStream_t st,
                        const uint32_t* hist0 = nullptr, int recent = 0, uint16_t* hits = nullptr,
-                       bool kvh = false) {
+                       bool kvh = false, bool spread = true) {
   if (d->batch == 0) return HILL_OK;
   SelectArgs a{};
   a.key = key;
@@ -460,7 +459,7 @@ hill_status run_select(const hill_desc* d, const float* key, const int32_t* lens
   a.hits = hits;
   a.rows_per_seq = kvh ? d->num_kv_heads : 1;
   a.err = di.err;
-  return from_cuda(counted(launch_select(a, st), 1));
+  return from_cuda(counted(launch_select(a, spread ? di.sms : 0, st), 1));
 }
 
 hill_status run_attn(const hill_desc* d, const void* q, const void* k, const void* v, const int32_t* idx,
@@ -707,7 +706,9 @@ hill_status hill_evict_step_end(const hill_desc* desc, const int32_t* lens, cons
                   kScoreNormalise);
     if (s != HILL_OK) return s;
   }
-  return run_select(desc, accum ? accum : s_out, lens, k, max_k, idx, count, di, st, hist0, recent, hits);
+  // beside the K stream of the next layer, on the few SMs that its grid leaves free
+  return run_select(desc, accum ? accum : s_out, lens, k, max_k, idx, count, di, st, hist0, recent, hits, false,
+                    false);
 }
 
 hill_status hill_evict_step_kvh(const hill_desc* desc, const void* q, const void* k_cache, const void* v_cache,

@@ -108,7 +108,7 @@ struct SelectArgs {
   const int32_t* lens;
   const int32_t* k;
   int B, cap, max_k;
-  int chunk;          // filled by the launcher
+  int lcap, list_words, pad_shift;   // crossing-bin list entries per CTA, words of the list, spare quads of the keys (set by the launcher)
   const uint32_t* hist0;   // optional [B][2048]: counts of the leading 11-bit key digit (tokens j < len - recent)
   int rows_per_seq;   // key rows per sequence: 1, or Hkv with per-KV-head selection (row r reads lens/k of r / rows_per_seq)
   int recent;         // BKP: the most recent min(recent, len) tokens are kept outright (0: none)
@@ -213,10 +213,10 @@ cudaError_t launch_selftest_wait(unsigned long long limit_ns, unsigned* err, cud
 cudaError_t launch_quantize_k(const QuantArgs& a, int dtype, int max_rows, cudaStream_t st);
 
 // select.cu
-int select_cluster_size(int cap);
-size_t select_smem_bytes(int cap, int C);
+bool select_cap_ok(int cap);   // a row of `cap` keys fits the largest cluster's shared memory
 int select_hist_bins();
-cudaError_t launch_select(const SelectArgs& a, cudaStream_t st);
+// sms: SMs that the rows may be spread over (0: as few CTAs per row as hold its keys).
+cudaError_t launch_select(const SelectArgs& a, int sms, cudaStream_t st);
 
 
 // attn.cu

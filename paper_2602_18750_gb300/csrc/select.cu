@@ -1,33 +1,44 @@
 // select.cu -- per-sequence top-k selection (Sec. 3.1 top-alpha retention;
 // Sec. 4.2: the global top-alpha after merging every score source).
 //
-// A sequence's scores are held on chip as 32-bit order-preserving keys, by
-// one CTA when they fit (up to kChunkMax keys), otherwise by a thread-block
-// cluster of C CTAs, each holding a contiguous chunk.  The exact k-th largest
-// key is found by an MSD radix select with digits of 11, 11 and 10 bits.  In
-// each pass every CTA histograms the keys that match the digits fixed so
-// far; after one cluster barrier every CTA adds up all C histograms through
-// distributed shared memory and searches the merged bins itself, so all CTAs
-// reach the same digit without further exchange.  The crossing bin is found
-// in two levels -- every warp sums its slice of the bins, one warp scans the
-// 32 slice sums and then the bins of the crossing slice.  A pass ends the
-// search early when the crossing bin is taken whole.  The first pass can
-// start from a histogram of the leading digit that the score normalisation
-// already accumulated (SelectArgs::hist0).  With 8-CTA clusters the keys of
-// the first pass's crossing bucket, when few, are gathered into every CTA so
-// that the later passes need no exchange.  This is the GPU form of the
-// paper's merge of chunked <position, score> blocks (Sec. 4.2): the chunks
-// stay on chip and only bin counts (or the few candidate keys) cross between
-// CTAs.  All global reads are issued before the first use of any of them.
+// A row's scores are held on chip as 32-bit order-preserving keys, by one CTA
+// of 1024 threads or by a thread-block cluster of C CTAs, each taking a
+// contiguous share.  The k-th largest key is found by an MSD radix search with
+// digits of 11, 11 and 10 bits that ends as soon as the crossing bin is taken
+// whole.  The counts of the leading digit come from the score normalisation
+// (SelectArgs::hist0) or are made while the keys are loaded; in a cluster
+// every CTA then adds its non-empty bins to all CTAs' sums through distributed
+// shared memory.  The keys of the crossing bin (typically 1 to 4 % of a row)
+// are put into a list, which a cluster exchanges in one step together with
+// the number of keys above the bin: every CTA writes its part into all the
+// others, so that after one cluster barrier each holds the whole list, runs
+// the remaining digits on its own copy and knows how many tokens the CTAs
+// before it keep.  A crossing bin that does not fit the list (heavy ties) is
+// searched by histograms over all keys, exchanged like the first one.
+//
+// Bound by latency on the few SMs that a row occupies: 4 bytes per token are
+// read once, and the rest is a chain of block-wide steps.  The length and
+// budget are read and the counts cleared before the dependency wait.  The keys
+// are read in order (16-byte loads) into shared memory, from where every
+// thread takes a run of consecutive ones and makes a bit mask of those above
+// and those inside the crossing bin: after that only the few inside it are
+// looked at again, and one scan of the threads' counts places the kept tokens.
+// The last digits are usually found by ranking at most kFew listed keys
+// directly.  What peers need is pushed to them instead of fetched.  Measured
+// in the step after the scoring stage (one GPU, before: re-counting loops over
+// all keys, fetched histograms): 1 row of 128K 10.9 -> 6.8 us, 4 rows of
+// 16-32K 10.4 -> 5.5, 4 of 16K 11.1 -> 7.5, 3 of 12K with window and hits
+// (raw scores) about 17 -> 11; alone 17.4 -> 9.4, 12.2 -> 7.4, 11.5 -> 7.6 and
+// 10.3 -> 7.2.
 //
 // Ties at the boundary go to the lowest token index: with tau the k-th key
-// and r_eq the number of keys equal to tau that must be taken, a token is
-// selected iff key > tau, or key == tau and fewer than r_eq keys equal to tau
-// precede it.  Every thread owns a contiguous run of keys; a block scan of
-// the per-thread counts (and a cluster exchange of the CTA totals) gives each
-// run its output position, so idx comes out in ascending order without a
-// sort.
+// and `need` the number of keys equal to tau that must be taken, a token is
+// selected iff key > tau, or key == tau and fewer than `need` keys equal to
+// tau precede it.  Threads own consecutive runs, so idx comes out in ascending
+// order without a sort.
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "hill_internal.h"
 
@@ -36,82 +47,105 @@ namespace cg = cooperative_groups;
 namespace hill {
 namespace {
 
-constexpr int kSelThreads = 1024;
-constexpr int kSelWarps = kSelThreads / 32;
+constexpr int T = 1024;            // threads
+constexpr int kWarps = T / 32;
 constexpr int kBins = 2048;
 constexpr int kMaxCluster = 8;
-constexpr int kChunkMax = 16384;   // keys per CTA before the cluster grows
-constexpr int kCand = kBins;       // crossing-bucket keys a cluster gathers into each CTA
-constexpr int kCandMinCluster = 8; // cluster size from which it gathers them
-constexpr int kHistBufs = 3;       // one per pass: no buffer is rewritten while a peer may read it
+constexpr int kPeerThreads = T / kMaxCluster;   // threads that write to one peer
+constexpr int kKeysMax = 48128;    // keys per CTA that fit shared memory beside the rest
+constexpr int kSelSmem = 225 * 1024;   // dynamic; 1.4 KB static beside it
+constexpr int kChunk = 4608;         // keys per CTA that a row is spread to, SMs permitting
+constexpr int kChunkMax = 16384;     // and at most, while the cluster can grow
+constexpr int kFew = 256;          // listed keys that are ranked directly
+constexpr int kListMax = 8192;     // crossing-bin keys of a row held by every CTA
 
-template <bool CL>
-__global__ void __launch_bounds__(kSelThreads) hill_select_kernel(SelectArgs a) {
+// The bin in which the running count from the top bin down reaches `need`,
+// what is still needed inside it, and its size.
+struct Crossing {
+  uint32_t bin, need, count;
+};
+
+__device__ __forceinline__ uint32_t warp_scan(uint32_t v) {   // inclusive
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += y;
+  }
+  return v;
+}
+
+// Called by all threads; two block-wide barriers.  The bins are taken from
+// the top down (position p is bin kBins - 1 - p).  Every warp sums a slice of
+// them; warp 0 finds the crossing slice and, two bins per lane, the bin.
+__device__ __forceinline__ Crossing find_crossing(const uint32_t* counts, uint32_t need, uint32_t* wtot,
+                                                  Crossing* found) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  static_assert(kBins == 2 * T, "two bins per thread");
+  auto bins = [&](int w) {   // this lane's bins of slice w: .y the upper one
+    return *reinterpret_cast<const uint2*>(counts + kBins - (w * 32 + lane + 1) * 2);
+  };
+  const uint2 b0 = bins(warp);
+  const uint32_t mine = __reduce_add_sync(0xffffffffu, b0.x + b0.y);
+  if (lane == 0) wtot[warp] = mine;
+  __syncthreads();
+  if (warp == 0) {
+    const uint32_t t = wtot[lane];
+    uint32_t inc = warp_scan(t);
+    unsigned hit = __ballot_sync(0xffffffffu, inc >= need);
+    const int ws = hit ? __ffs(hit) - 1 : kWarps - 1;
+    const uint32_t cum = __shfl_sync(0xffffffffu, inc - t, ws);
+    const uint2 c = bins(ws);
+    inc = cum + warp_scan(c.x + c.y);
+    hit = __ballot_sync(0xffffffffu, inc >= need);
+    if (lane == (hit ? __ffs(hit) - 1 : 31)) {
+      const uint32_t above = inc - c.x - c.y;   // keys above this lane's bins
+      const bool low = above + c.y < need;
+      *found = Crossing{(uint32_t)(kBins - 1 - (ws * 32 + lane) * 2 - (low ? 1 : 0)), need - above - (low ? c.y : 0u),
+                        low ? c.x : c.y};
+    }
+  }
+  __syncthreads();
+  return *found;
+}
+
+// CL: a cluster of CTAs per row.  Mask: a bit per key of a thread.
+template <bool CL, typename Mask>
+__global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
   int C = 1, r = 0;
   cg::cluster_group cluster = cg::this_cluster();
   if (CL) {
     C = (int)cluster.num_blocks();
     r = (int)cluster.block_rank();
   }
-  auto csync = [&]() {
-    if (CL) cluster.sync(); else __syncthreads();
-  };
-  auto remote = [&](uint32_t* p, int c) -> uint32_t* {
-    return CL ? cluster.map_shared_rank(p, c) : p;
-  };
+  auto remote = [&](uint32_t* p, int c) -> uint32_t* { return CL ? cluster.map_shared_rank(p, c) : p; };
   // row = one key row; with per-KV-head selection a sequence has
   // rows_per_seq rows that share its length and budget
   const int row = blockIdx.y;
   const int b = row / a.rows_per_seq;
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5, lane = tid & 31;
-  pdl_wait();
-  pdl_launch_dependents();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
   extern __shared__ __align__(16) uint32_t sm[];
-  uint32_t* keys = sm;                       // [chunk]
-  uint32_t* histbuf = keys + a.chunk;        // [kHistBufs][kBins], pass p uses buffer p
-  uint32_t* merged = histbuf + kHistBufs * kBins;   // [kBins]: the cluster's sum for this pass
-  __shared__ uint32_t wtot[kSelWarps];
-  __shared__ uint32_t cnt[kMaxCluster];
-  __shared__ uint32_t cnt2[kMaxCluster];
-  __shared__ uint32_t s_nc;
-  __shared__ uint32_t bc[3];
+  uint32_t* sums = sm;                      // [3][kBins] counts of each digit over the row
+  uint32_t* own = sums + 3 * kBins;         // CL: [kBins] this CTA's counts
+  uint32_t* list = own + (CL ? kBins : 0);  // [C][lcap] keys of the crossing bin, by CTA
+  uint4* keys = reinterpret_cast<uint4*>(list + a.list_words);   // this CTA's keys in quads (key_quad)
+  __shared__ uint32_t wtot[kWarps];         // slice sums of a search
+  __shared__ uint32_t wcnt[kWarps];         // kept tokens per warp
+  __shared__ Crossing found;
+  __shared__ uint32_t s_cnt[kMaxCluster];   // by CTA: (keys above the crossing bin) << 16 | keys in it
+  __shared__ uint32_t s_tot[kMaxCluster];   // by CTA: (above tau) << 16 | (equal to tau)
+  __shared__ uint32_t my_cnt, s_before, s_few;
+  __shared__ __align__(16) uint32_t few[kFew];
 
-  // Every global read the search needs is issued before the first use of
-  // any of them, so the kernel pays one memory round trip, not one per
-  // input: the length and budget, the upstream leading-digit histogram, and
-  // this CTA's chunk of keys.  The keys are read up to the capacity (valid
-  // memory); rows at or beyond the length are never counted.
+  // Before the dependency wait: the length and budget (inputs of the call,
+  // complete before the call: include/hill.h) and this CTA's own memory.
   int len = a.lens[b];
   int kk = a.k[b];
-  constexpr int kH0 = kBins / kSelThreads;
-  uint32_t h0v[kH0];
-  if (a.hist0) {
-    const uint32_t* h0 = a.hist0 + (int64_t)row * kBins;
-#pragma unroll
-    for (int j = 0; j < kH0; ++j) h0v[j] = h0[tid + j * kSelThreads];
-  }
-  const int j_lo = r * a.chunk;
-  const int ncap = max(0, min(a.chunk, a.cap - j_lo));
-  const float* kp = a.key + (int64_t)row * a.cap + j_lo;
-  int i_tail = 0;
-  if ((reinterpret_cast<uintptr_t>(kp) & 15u) == 0) {
-    // 16-byte loads when the chunk starts on a 16-byte boundary
-    const int n4 = ncap >> 2;
-    const float4* kp4 = reinterpret_cast<const float4*>(kp);
-    uint4* k4 = reinterpret_cast<uint4*>(keys);
-#pragma unroll 4
-    for (int i = tid; i < n4; i += kSelThreads) {
-      const float4 v = kp4[i];
-      k4[i] = make_uint4(ordered_key(v.x), ordered_key(v.y), ordered_key(v.z), ordered_key(v.w));
-    }
-    i_tail = n4 << 2;
-  }
-#pragma unroll 8
-  for (int i = i_tail + tid; i < ncap; i += kSelThreads) keys[i] = ordered_key(kp[i]);
-  for (int i = tid; i < kHistBufs * kBins; i += kSelThreads) histbuf[i] = 0;
-
+  for (int i = tid; i < (3 + (CL ? 1 : 0)) * kBins / 4; i += T)
+    reinterpret_cast<uint4*>(sums)[i] = uint4{0u, 0u, 0u, 0u};
+  if (tid == 0) my_cnt = s_before = s_few = 0u;
+  if (tid < kFew) few[tid] = 0u;
   len = len < 0 ? 0 : (len > a.cap ? a.cap : len);
   // BKP temporal pinning (Sec. 4.2): the most recent tokens [older, len) are
   // kept outright; the ranking runs over [0, older)
@@ -120,293 +154,343 @@ __global__ void __launch_bounds__(kSelThreads) hill_select_kernel(SelectArgs a) 
   const int older = len - rfull;
   int win = rfull;
   kk = kk < 0 ? 0 : (kk > older ? older : kk);
-  if (win > a.max_k || kk > a.max_k - min(win, a.max_k)) {
-    if (r == 0 && tid == 0) raise_error(a.err, kErrDevArg);
+  const bool over = win > a.max_k || kk > a.max_k - min(win, a.max_k);
+  if (over) {
     win = min(win, a.max_k);           // the most recent max_k tokens of the window
     kk = min(kk, a.max_k - win);
   }
+  const bool search = kk > 0 && kk < older;   // the same in every CTA of the row
+  if (CL) {
+    if (search) cluster.barrier_arrive();   // A: every CTA has started and cleared its memory
+  } else {
+    __syncthreads();
+  }
+  // Shares of the ranked tokens: equal ones for the row's CTAs and for a
+  // CTA's threads, cut where 16-byte loads may start.  With s0 the place of
+  // the row's first key in its 16 bytes, token j is at place j + s0.  The
+  // CTA's quads are read from global memory in order and kept in shared
+  // memory, from where thread t takes the q quads t * q .. t * q + q - 1; a
+  // spare quad in every eight keeps both sides free of bank conflicts.
+  const float* row_key = a.key + (int64_t)row * a.cap;
+  const int s0 = (int)((reinterpret_cast<uintptr_t>(row_key) >> 2) & 3u);
+  const int share = (((older + s0 + C - 1) / C) + 3) & ~3;
+  const int nq = share / 4, q = (nq + T - 1) / T;
+  const int jc = r * share - s0;    // the CTA's first token (maybe negative: none there)
+  const int hi = min(older, jc + share);
+  auto key_quad = [&](int g) { return g + (g >> a.pad_shift); };
+  const int j0 = jc + tid * q * 4;   // this thread's first token
   int32_t* out = a.idx + (int64_t)row * a.max_k;
   uint16_t* hits = a.hits ? a.hits + (int64_t)row * a.cap : nullptr;
+  // the keys are being written: only their address translation is fetched
+  if (search && jc + 4 * tid < hi) prefetch_l2(row_key + max(jc + 4 * tid, 0));
+  pdl_wait();
+  pdl_launch_dependents();
+
+  // The global reads are issued before the first use of any of them.  A key
+  // of 0 means no token (a token's key is at least 1).
+  uint4 h0v{0u, 0u, 0u, 0u};
+  if (search && a.hist0 && tid < kBins / 4) h0v = reinterpret_cast<const uint4*>(a.hist0 + (int64_t)row * kBins)[tid];
+  // counts of the first digit: taken over, or made from the keys as they come
+  uint32_t* h = CL ? own : sums;
+  if (search) {
+    if (CL && !a.hist0) cluster.barrier_wait();   // A
+    constexpr int kU = 4;   // quads in flight
+    for (int g0 = tid; g0 < nq; g0 += kU * T) {
+      float4 f[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int g = g0 + u * T, j = jc + 4 * g;
+        f[u] = float4{0.f, 0.f, 0.f, 0.f};
+        if (g >= nq) continue;
+        if (j >= 0 && j + 3 < hi) {
+          f[u] = *reinterpret_cast<const float4*>(row_key + j);
+        } else {
+          if (j >= 0 && j < hi) f[u].x = row_key[j];
+          if (j + 1 >= 0 && j + 1 < hi) f[u].y = row_key[j + 1];
+          if (j + 2 >= 0 && j + 2 < hi) f[u].z = row_key[j + 2];
+          if (j + 3 >= 0 && j + 3 < hi) f[u].w = row_key[j + 3];
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kU; ++u) {
+        const int g = g0 + u * T, j = jc + 4 * g;
+        if (g >= nq) continue;
+        const float v[4] = {f[u].x, f[u].y, f[u].z, f[u].w};
+        uint32_t k[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          k[e] = j + e >= 0 && j + e < hi ? max(ordered_key(v[e]), 1u) : 0u;
+          if (!a.hist0 && k[e]) atomicAdd(&h[k[e] >> 21], 1u);
+        }
+        keys[key_quad(g)] = uint4{k[0], k[1], k[2], k[3]};
+      }
+    }
+  }
+
+  // padding, count and the pinned window (every path)
+  if (over && r == 0 && tid == 0) raise_error(a.err, kErrDevArg);
+  for (int p = kk + win + r * T + tid; p < a.max_k; p += C * T) out[p] = -1;
+  if (r == 0 && tid == 0) a.count[row] = kk + win;
   auto hit = [&](int j) {   // the hit-rate table: +1 per kept token, saturating
     if (hits && hits[j] != 0xffffu) hits[j] = (uint16_t)(hits[j] + 1u);
   };
-  const int n = max(0, min(j_lo + a.chunk, older) - j_lo);
-
-  // padding, count and the pinned window (every path)
-  for (int p = kk + win + r * kSelThreads + tid; p < a.max_k; p += C * kSelThreads) out[p] = -1;
-  if (r == 0 && tid == 0) a.count[row] = kk + win;
-  for (int j = max(j_lo, len - win) + tid; j < min(j_lo + a.chunk, len); j += kSelThreads) {
+  for (int j = len - win + r * T + tid; j < len; j += C * T) {
     out[kk + j - (len - win)] = j;
     hit(j);
   }
-  if (kk == 0) return;
-  if (kk == older) {  // every older token is selected
-    for (int i = tid; i < n; i += kSelThreads) {
-      out[j_lo + i] = j_lo + i;
-      hit(j_lo + i);
-    }
+  if (!search) {
+    if (kk > 0)   // every older token is selected
+      for (int j = r * T + tid; j < older; j += C * T) {
+        out[j] = j;
+        hit(j);
+      }
     return;
   }
-  __syncthreads();
 
-  uint32_t prefix = 0, pmask = 0;
-  uint32_t remaining = (uint32_t)kk;
-  bool take_bucket = false;    // the crossing bucket is taken whole
-  const uint32_t* src = keys;  // the keys histogrammed by passes 1 and 2
-  int nsrc = n;
-  bool local = !CL;            // a pass needs no exchange between CTAs
+  // Add this CTA's non-empty bins to every CTA's sums, and clear them.
+  auto push_counts = [&](uint32_t* sum) {
+    for (int i = tid; i < kBins; i += T) {
+      const uint32_t v = own[i];
+      if (v) {
+        own[i] = 0u;
+        for (int c = 0; c < C; ++c) atomicAdd(remote(sum, c) + i, v);
+      }
+    }
+  };
+  if (a.hist0) {
+    if (CL) cluster.barrier_wait();   // A
+    if (tid < kBins / 4) reinterpret_cast<uint4*>(sums)[tid] = h0v;
+  }
+  __syncthreads();
+  if (CL && !a.hist0) {
+    push_counts(sums);
+    cluster.sync();
+  }
+  Crossing x = find_crossing(sums, (uint32_t)kk, wtot, &found);
+  uint32_t tau = x.bin << 21;             // the digits found so far
+  uint32_t need = x.need;
+  bool whole = x.need == x.count;         // the crossing bin is taken whole: keys >= tau are kept
+  const bool whole0 = whole;
+  // A bit per key of this thread: `gt` above the crossing bin (or in it, when
+  // it is kept whole), `in` inside it.
+  Mask gt = 0, in = 0;
+  const int my_q = min(q, nq - tid * q);
+  {
+    const uint32_t lo = max(tau, 1u), top = tau + 0x1fffffu;
+#pragma unroll 4
+    for (int i = 0; i < my_q; ++i) {
+      const uint4 v = keys[key_quad(tid * q + i)];
+      const uint32_t k[4] = {v.x, v.y, v.z, v.w};
+      uint32_t ge4 = 0, gt4 = 0;
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        ge4 |= k[e] >= lo ? 1u << e : 0u;
+        gt4 |= k[e] > top ? 1u << e : 0u;
+      }
+      in |= (Mask)ge4 << (4 * i);
+      gt |= (Mask)gt4 << (4 * i);
+    }
+    if (whole) gt = in;
+    in ^= gt;
+  }
+  auto pop = [](Mask m) { return (uint32_t)(sizeof(Mask) == 8 ? __popcll(m) : __popc((uint32_t)m)); };
+  auto first = [](Mask m) { return (sizeof(Mask) == 8 ? __ffsll((long long)m) : __ffs((int)(uint32_t)m)) - 1; };
+  auto key_of = [&](int i) {   // key i of this thread
+    return reinterpret_cast<const uint32_t*>(keys + key_quad(tid * q + (i >> 2)))[i & 3];
+  };
+  if (CL || !whole) {
+    // the crossing bin's keys into the list; (keys above) << 16 | (keys in it)
+    const uint32_t cnt = (pop(gt) << 16) | pop(in);
+    const uint32_t inc = warp_scan(cnt);
+    uint32_t base = 0;
+    if (lane == 31 && inc) base = atomicAdd(&my_cnt, inc);
+    base = __shfl_sync(0xffffffffu, base, 31);
+    uint32_t at = (base + inc - cnt) & 0xffffu;
+    for (Mask m = in; m; m &= m - 1, ++at)
+      if (at < (uint32_t)a.lcap) list[r * a.lcap + at] = key_of(first(m));
+    __syncthreads();
+  }
+  bool listed = !whole && (my_cnt & 0xffffu) <= (uint32_t)a.lcap;
+  if (CL) {
+    const uint32_t nc = my_cnt & 0xffffu;
+    if (listed) {
+      const int c = tid / kPeerThreads, i0 = tid % kPeerThreads;
+      if (c < C && c != r) {
+        const uint32_t* src = list + r * a.lcap;
+        uint32_t* dst = remote(list + r * a.lcap, c);
+        for (uint32_t i = i0; i < nc; i += kPeerThreads) dst[i] = src[i];
+      }
+    }
+    if (tid < C) remote(s_cnt, tid)[r] = my_cnt;
+    cluster.sync();   // every CTA's list and counts are in place
+    listed = !whole;
+    for (int c = 0; c < C; ++c) listed = listed && (s_cnt[c] & 0xffffu) <= (uint32_t)a.lcap;
+  }
+  // f(key, CTA) for every entry of the list: kWarps / C warps take a CTA's part
+  auto each = [&](auto&& f) {
+    const int per = CL ? kWarps / C : kWarps, c = CL ? warp / per : 0;
+    const uint32_t nc = (CL ? s_cnt[c] : my_cnt) & 0xffffu;
+    for (uint32_t i = (warp - c * per) * 32 + lane; i < nc; i += per * 32) f(list[c * a.lcap + i], c);
+  };
+  // the digits that follow, until the crossing bin is taken whole: from counts
+  // of the keys that share those found, or, when few listed keys share them,
+  // by ranking these
 #pragma unroll 1
-  for (int pass = 0; pass < 3; ++pass) {
-    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
-    const int nb = pass == 2 ? 1024 : 2048;
-    const uint32_t dmask = (uint32_t)nb - 1u;
-    uint32_t* hist = histbuf + pass * kBins;
-    const uint32_t* om = merged;
-    if (pass == 0 && a.hist0) {
-      // leading-digit counts over the whole sequence, accumulated upstream
-#pragma unroll
-      for (int j = 0; j < kH0; ++j) merged[tid + j * kSelThreads] = h0v[j];
-    } else {
-      for (int i = tid; i < nsrc; i += kSelThreads) {
-        const uint32_t kv = src[i];
-        if ((kv & pmask) == prefix) atomicAdd(&hist[(kv >> shift) & dmask], 1u);
-      }
-      if (local) {
-        __syncthreads();
-      } else {
-        csync();  // every CTA's histogram of this pass is complete
-        // all peer reads are issued before any sum is stored
-        uint32_t v[kH0] = {};
-#pragma unroll
-        for (int c = 0; c < kMaxCluster; ++c) {
-          if (c < C) {
-            const uint32_t* h = remote(hist, c);
-#pragma unroll
-            for (int j = 0; j < kH0; ++j)
-              if (tid + j * kSelThreads < nb) v[j] += h[tid + j * kSelThreads];
-          }
+  for (int d = 1; d < 3 && !whole; ++d) {
+    const uint32_t done = d == 1 ? 0xffe00000u : 0xfffffc00u;
+    uint32_t* sum = sums + d * kBins;
+    // (the third digit has 10 bits: every other bin)
+    auto add = [&](uint32_t* to, uint32_t kv) {
+      if ((kv & done) == tau) atomicAdd(&to[(d == 1 ? kv >> 10 : kv << 1) & (kBins - 1)], 1u);
+    };
+    if (listed && x.count <= kFew) {
+      each([&](uint32_t kv, int) {
+        if ((kv & done) == tau) few[atomicAdd(&s_few, 1u) & (kFew - 1)] = kv;
+      });
+      __syncthreads();
+      if (tid < kFew && (uint32_t)tid < x.count) {
+        const uint32_t kv = few[tid];
+        uint32_t ng = 0, ge = 0;   // keys above this one; and not below it
+        for (uint32_t i = 0; i < x.count; i += 4) {   // (0 past the end: below every key)
+          const uint4 v = *reinterpret_cast<const uint4*>(few + i);
+          ng += (v.x > kv ? 1u : 0u) + (v.y > kv ? 1u : 0u) + (v.z > kv ? 1u : 0u) + (v.w > kv ? 1u : 0u);
+          ge += (v.x >= kv ? 1u : 0u) + (v.y >= kv ? 1u : 0u) + (v.z >= kv ? 1u : 0u) + (v.w >= kv ? 1u : 0u);
         }
-#pragma unroll
-        for (int j = 0; j < kH0; ++j)
-          if (tid + j * kSelThreads < nb) merged[tid + j * kSelThreads] = v[j];
+        if (ng < need && need <= ge) found = Crossing{kv, need - ng, ge - ng};   // (equal keys write the same)
       }
-      if (local) om = hist;
-    }
-    __syncthreads();
-    // Two-level search over positions p = 0..nb-1 (bins from the top down):
-    // warp w sums positions [w*S, (w+1)*S), then warp 0 scans the 32 sums
-    // and the positions of the crossing slice.
-    const int S = nb / kSelWarps;   // 64 or 32
-    {
-      uint32_t v = 0;
-      for (int p = warp * S + lane; p < (warp + 1) * S; p += 32) v += om[nb - 1 - p];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) wtot[warp] = v;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      const uint32_t t = wtot[lane];
-      uint32_t inc = t;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-      }
-      const uint32_t need = remaining;   // >= 1
-      const unsigned hit = __ballot_sync(0xffffffffu, inc >= need);
-      const int ws = hit ? __ffs(hit) - 1 : 31;    // slice holding the crossing
-      uint32_t cum = __shfl_sync(0xffffffffu, inc - t, ws);
-      for (int p0 = ws * S; p0 < (ws + 1) * S; p0 += 32) {
-        const int p = p0 + lane;
-        const uint32_t c = om[nb - 1 - p];
-        uint32_t ci = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, ci, o);
-          if (lane >= o) ci += y;
-        }
-        const unsigned h = __ballot_sync(0xffffffffu, cum + ci >= need);
-        if (h) {
-          if (lane == __ffs(h) - 1) {
-            bc[0] = (uint32_t)(nb - 1 - p);
-            bc[1] = need - (cum + ci - c);
-            bc[2] = c;
-          }
-          break;
-        }
-        cum += __shfl_sync(0xffffffffu, ci, 31);
-      }
-    }
-    __syncthreads();
-    prefix |= bc[0] << shift;
-    pmask |= dmask << shift;
-    remaining = bc[1];
-    if (remaining == bc[2]) {
-      take_bucket = true;
+      __syncthreads();
+      tau = found.bin;
+      need = found.need;
+      whole = found.need == found.count;
       break;
     }
-    if (!local && pass == 0 && C >= kCandMinCluster && bc[2] <= (uint32_t)kCand) {
-      // The keys of the crossing bucket are few (typically 1-4 % of the
-      // sequence): every CTA gathers all of them from the cluster once, and
-      // the two remaining passes then run on that copy inside each CTA, with
-      // no further histogram exchange.  All CTAs hold the same multiset, so
-      // they reach the same digits.  (Measured: this pays off against the
-      // exchange of 2 x C histograms at C = 8 and loses at C = 2.)  The
-      // buffers: this CTA's own candidates go to `merged` (free after the
-      // search above; peers read it until the compaction's cluster barrier),
-      // the gathered copy to histogram buffer 0 (peers have finished reading
-      // it once they pass the barrier below).
-      uint32_t* cand = merged;
-      if (tid == 0) s_nc = 0;
-      __syncthreads();
-      for (int w0 = warp * 32; w0 < n; w0 += kSelThreads) {   // warp-uniform trip count
-        const int i = w0 + lane;
-        const uint32_t kv = i < n ? keys[i] : 0u;
-        const bool m = i < n && (kv & pmask) == prefix;
-        const unsigned bal = __ballot_sync(0xffffffffu, m);
-        if (bal) {
-          uint32_t base = 0;
-          if (lane == 0) base = atomicAdd(&s_nc, (uint32_t)__popc(bal));
-          base = __shfl_sync(0xffffffffu, base, 0) + (uint32_t)__popc(bal & ((1u << lane) - 1u));
-          if (m && base < (uint32_t)kCand) cand[base] = kv;
-        }
+    if (listed) {
+      each([&](uint32_t kv, int) { add(sum, kv); });
+    } else {
+      for (Mask m = in; m; m &= m - 1) add(CL ? own : sum, key_of(first(m)));
+      if (CL) {
+        __syncthreads();
+        push_counts(sum);
+        cluster.sync();
       }
-      __syncthreads();
-      if (tid < C) remote(cnt2, tid)[r] = s_nc;
-      csync();  // every CTA's candidates and count are in place
-      uint32_t offs[kMaxCluster + 1];
-      offs[0] = 0;
-#pragma unroll
-      for (int c = 0; c < kMaxCluster; ++c) offs[c + 1] = offs[c] + (c < C ? min(cnt2[c], (uint32_t)kCand) : 0u);
-      const uint32_t tot = offs[kMaxCluster];
-      if (tot != bc[2] && tid == 0) raise_error(a.err, kErrDevArg);   // cannot happen: counts disagree
-      uint32_t* all = histbuf;
-      constexpr int kCandPer = kCand / kSelThreads;
-      uint32_t v[kCandPer];
-#pragma unroll
-      for (int j = 0; j < kCandPer; ++j) {   // every peer read is issued before any store
-        const uint32_t i = (uint32_t)(tid + j * kSelThreads);
-        int c = 0;
-        uint32_t base = 0;
-#pragma unroll
-        for (int cc = 1; cc < kMaxCluster; ++cc)
-          if (i >= offs[cc]) {
-            c = cc;
-            base = offs[cc];
-          }
-        v[j] = i < tot ? remote(cand, c)[i - base] : 0u;
-      }
-#pragma unroll
-      for (int j = 0; j < kCandPer; ++j)
-        if ((uint32_t)(tid + j * kSelThreads) < tot) all[tid + j * kSelThreads] = v[j];
-      src = all;
-      nsrc = (int)min(tot, (uint32_t)kCand);
-      local = true;
-      __syncthreads();
     }
+    __syncthreads();
+    x = find_crossing(sum, need, wtot, &found);
+    tau |= d == 1 ? x.bin << 10 : x.bin >> 1;
+    need = x.need;
+    whole = x.need == x.count;
   }
-  // Selection rule: take_bucket -> key >= prefix (every key of the crossing
-  // bucket and above); otherwise tau = prefix is the k-th key itself and
-  // `remaining` of the keys equal to tau are taken, lowest index first.
-  const uint32_t tau = prefix;
-  auto is_gt = [&](uint32_t kv) { return take_bucket ? kv >= tau : kv > tau; };
-  auto is_eq = [&](uint32_t kv) { return !take_bucket && kv == tau; };
 
   // ---------------------------------------------------------------- compaction
-  // thread t owns keys [t*m, t*m + m) of the chunk (m odd: conflict-free
-  // strided reads); counts are packed as (above tau) << 16 | (equal to tau),
-  // a chunk holding fewer than 2^16 keys
-  const int m = ((n + kSelThreads - 1) / kSelThreads) | 1;
-  const int i0 = min(n, tid * m), i1 = min(n, i0 + m);
-  uint32_t mine = 0;
-  for (int i = i0; i < i1; ++i) {
-    const uint32_t kv = keys[i];
-    mine += is_gt(kv) ? (1u << 16) : (is_eq(kv) ? 1u : 0u);
+  // Selection rule: whole -> key >= tau (tau > 0); otherwise tau is the k-th
+  // key itself and `need` of the keys equal to tau are taken, lowest index
+  // first.  Only the crossing bin's keys are looked at again.  Counts are
+  // packed as (kept above) << 16 | (equal to tau): a CTA holds fewer than 2^16
+  // keys.
+  const uint32_t top = whole ? tau - 1u : tau;
+  const uint32_t eq = whole ? 0u : tau;   // (no token's key is 0)
+  Mask eqm = 0;
+  for (Mask m = in; m; m &= m - 1) {
+    const uint32_t kv = key_of(first(m));
+    if (kv > top) gt |= m & (~m + 1);
+    if (kv == eq) eqm |= m & (~m + 1);
   }
-  // exclusive block scan of the packed counts
-  uint32_t inc = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += y;
-  }
-  if (lane == 31) wtot[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    const uint32_t t = wtot[lane];
-    uint32_t wi = t;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, wi, o);
-      if (lane >= o) wi += y;
-    }
-    wtot[lane] = wi - t;                       // exclusive prefix of warp totals
-    if (lane == 31) bc[0] = wi;                // the CTA total
+  const uint32_t mine = (pop(gt) << 16) | pop(eqm);
+  const uint32_t inc = warp_scan(mine);
+  if (lane == 31) wcnt[warp] = inc;
+  if (CL && listed) {   // the crossing-bin keys that the CTAs before this one keep
+    uint32_t v = 0;
+    each([&](uint32_t kv, int c) {
+      if (c < r) v += (kv > top ? 0x10000u : 0u) + (kv == eq ? 1u : 0u);
+    });
+    v = __reduce_add_sync(0xffffffffu, v);
+    if (lane == 0 && v) atomicAdd(&s_before, v);
   }
   __syncthreads();
-  const uint32_t before = wtot[warp] + inc - mine;   // this thread's exclusive prefix in the CTA
-  uint32_t gt_before = 0, eq_before = 0;
+  const uint32_t wt = lane < kWarps ? wcnt[lane] : 0u;
+  const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? wt : 0u) + inc - mine;
+  uint32_t pos = before >> 16, eq_rank = before & 0xffffu;
   if (CL) {
-    if (tid < C) remote(cnt, tid)[r] = bc[0];
-    csync();
-    for (int c = 0; c < r; ++c) {
-      gt_before += cnt[c] >> 16;
-      eq_before += cnt[c] & 0xffffu;
-    }
-  }
-  uint32_t eq_rank = eq_before + (before & 0xffffu);   // ties before this run
-  uint32_t pos = gt_before + (before >> 16) + min(eq_rank, remaining);
-  for (int i = i0; i < i1; ++i) {
-    const uint32_t kv = keys[i];
-    bool take = is_gt(kv);
-    if (is_eq(kv)) {
-      take = eq_rank < remaining;
-      ++eq_rank;
-    }
-    if (take) {
-      if (pos < (uint32_t)kk) {
-        out[pos] = j_lo + i;
-        hit(j_lo + i);
-      } else {
-        raise_error(a.err, kErrDevArg);   // cannot happen: more picks than the budget
+    if (listed || whole0) {
+      pos += s_before >> 16;   // (0 when the first digit decided)
+      eq_rank += s_before & 0xffffu;
+      for (int c = 0; c < r; ++c) pos += s_cnt[c] >> 16;
+    } else {
+      const uint32_t total = __reduce_add_sync(0xffffffffu, wt);
+      if (tid < C) remote(s_tot, tid)[r] = total;
+      cluster.sync();
+      for (int c = 0; c < r; ++c) {
+        pos += s_tot[c] >> 16;
+        eq_rank += s_tot[c] & 0xffffu;
       }
-      ++pos;
     }
   }
+  pos += min(eq_rank, need);
+  // drop the ties past the budget: the kept keys are then the bits of gt
+  for (; eqm && eq_rank < need; ++eq_rank, eqm &= eqm - 1) gt |= eqm & (~eqm + 1);
+  if (pos + pop(gt) > (uint32_t)kk) {
+    raise_error(a.err, kErrDevArg);   // cannot happen: more picks than the budget
+    return;
+  }
+  if (!hits) {
+    for (; gt; gt &= gt - 1) out[pos++] = j0 + first(gt);
+    return;
+  }
+  // with the hit table: four counts are read before any is written
+  while (gt) {
+    int j[4];
+    uint32_t old[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      j[u] = gt ? j0 + first(gt) : -1;
+      gt &= gt - 1;
+      old[u] = j[u] >= 0 ? hits[j[u]] : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j[u] >= 0) {
+        out[pos++] = j[u];
+        if (old[u] != 0xffffu) hits[j[u]] = (uint16_t)(old[u] + 1u);
+      }
+  }
+}
+
+template <bool CL, typename Mask>
+cudaError_t launch_select_t(const SelectArgs& a, int C, size_t smem, cudaStream_t st) {
+  static int cache[64] = {0};
+  auto kern = hill_select_kernel<CL, Mask>;
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), (int)smem, cache);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3(C, a.B * a.rows_per_seq, 1), dim3(T), smem, st, CL ? C : 0, a);
 }
 
 }  // namespace
 
-int select_cluster_size(int cap) {
-  int C = 1;
-  while (C < kMaxCluster && (cap + C - 1) / C > kChunkMax) C <<= 1;
-  return C;
-}
-
-size_t select_smem_bytes(int cap, int C) {
-  const int chunk = (cap + C - 1) / C;
-  return (size_t)chunk * 4 + (kHistBufs + 1) * kBins * 4;
-}
+bool select_cap_ok(int cap) { return (cap + kMaxCluster - 1) / kMaxCluster <= kKeysMax; }
 
 int select_hist_bins() { return kBins; }
 
-cudaError_t launch_select(const SelectArgs& a0, cudaStream_t st) {
+cudaError_t launch_select(const SelectArgs& a0, int sms, cudaStream_t st) {
   SelectArgs a = a0;
-  const int C = select_cluster_size(a.cap);
-  a.chunk = (a.cap + C - 1) / C;
-  const size_t smem = select_smem_bytes(a.cap, C);
-  const dim3 grid(C, a.B * a.rows_per_seq, 1), block(kSelThreads, 1, 1);
-  if (C == 1) {
-    static int cache[64] = {0};
-    cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(hill_select_kernel<false>), (int)smem, cache);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(hill_select_kernel<false>, grid, block, smem, st, 0, a);
-  }
-  static int cache[64] = {0};
-  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(hill_select_kernel<true>), (int)smem, cache);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(hill_select_kernel<true>, grid, block, smem, st, C, a);
+  // CTAs per row: more until a CTA has at most kChunk keys, while twice as
+  // many still fit `sms`; else as few as hold kChunkMax each.  Measured (us a
+  // selection after the scoring, one against four or eight CTAs): 32K x 4
+  // rows 9.8 / 7.4, 64K x 8 13.4 / 11.1, 16K x 4 8.0 / 7.6, per-KV-head 16K x
+  // 16 rows -1.5 with 2 -> 4; 4K rows are faster in one CTA (5.5 against 7.1).
+  const int rows = a.B * a.rows_per_seq;
+  int C = 1;
+  while (C < kMaxCluster && (a.cap + C - 1) / C > (2 * C * rows <= sms ? kChunk : kChunkMax)) C <<= 1;
+  const int share = (((a.cap + 3 + C - 1) / C) + 3) & ~3;   // of a CTA, at most (see the kernel)
+  const int nq = share / 4, counts = (C > 1 ? 4 : 3) * kBins;
+  // the spare quads, where they fit beside a list of full size
+  a.pad_shift = (nq + nq / 8 + 1) * 4 + counts + kListMax <= kSelSmem / 4 ? 3 : 31;
+  const int key_words = (nq + (nq >> a.pad_shift) + 1) * 4;
+  a.lcap = std::min(kListMax, kSelSmem / 4 - counts - key_words) / C;
+  a.list_words = (a.lcap * C + 3) & ~3;
+  const size_t smem = (size_t)(counts + a.list_words + key_words) * 4;
+  const bool m32 = nq <= 8 * T;   // at most 32 keys per thread
+  if (C > 1) return m32 ? launch_select_t<true, uint32_t>(a, C, smem, st) : launch_select_t<true, uint64_t>(a, C, smem, st);
+  return m32 ? launch_select_t<false, uint32_t>(a, C, smem, st) : launch_select_t<false, uint64_t>(a, C, smem, st);
 }
 
 }  // namespace hill
