@@ -26,7 +26,7 @@ struct ScoreArgs {
   float* accum;       // RAW: running importance (+=), may be NULL
   float* logits;      // ATTN: [B][H][lstride] (lstride = cap rounded up to 32: a warp's 32 tokens of a head fill one 128-byte line)
   int64_t lstride;
-  float2* partials;   // ATTN: [B][nslot][H] (max, sum 2^(z2 - max)), base-2 logits z2 = z * log2 e
+  float2* partials;   // ATTN: [B][H][nslot] (max, sum 2^(z2 - max)), base-2 logits z2 = z * log2 e
   int nslot;          // = grid size of the launch x score_deal_warps(nkv, G) (one slot per warp share)
   int kvh;            // RAW with per-KV-head selection: scores/accum [B][Hkv][cap], summed over each group only
   // Query heads per KV head in the data (Gs), the first one this launch
@@ -55,8 +55,8 @@ struct FinalizeArgs {
   int recent;         // tokens j >= len - min(recent, len) are left out of hist0 (pinned, not ranked)
   int kvh;            // 1: scores/accum are [B][Hkv][cap], the sum over each KV head's G query heads
   int Hkv;
-  float2* stats;      // [B][H] (max, 1/sum) per head, or NULL: every finalize CTA combines the partials
-  int tpt;            // blocks of 256 tokens per finalize CTA (set by the launcher)
+  float2* stats;      // [B][H] (max, 1/sum) per head, written by hill_attn_stats_kernel in the split step
+  int tpt;            // blocks of tokens per finalize CTA (set by the launcher)
 };
 
 // The E4M3 scoring on the tensor cores' native 8-bit path (score_tc.cu):
@@ -75,7 +75,7 @@ struct ScoreTcArgs {
   float* accum;       // RAW: running importance (+=), may be NULL
   float* logits;      // ATTN: [B][H][lstride]
   int64_t lstride;
-  float2* partials;   // ATTN: [B][nslot][H] (max, sum 2^(z2 - max)), one slot per CTA meeting the sequence
+  float2* partials;   // ATTN: [B][H][nslot] (max, sum 2^(z2 - max)), one slot per CTA meeting the sequence
   int nslot;
   uint32_t* hist0;    // optional: zero-filled here for the normalisation to count into
   int64_t hist0_words;

@@ -26,10 +26,9 @@
 //         own tokens per head in registers, and the lanes of a head are
 //         combined once, when the CTA leaves a sequence, into one partial per
 //         (sequence, head, CTA).  hill_attn_finalize_kernel combines the
-//         partials and forms s[b,j] = sum_h exp(z[b,h,j] - m_bh) / L_bh; when
-//         that kernel would need more than two CTAs per SM (long sequences),
-//         hill_attn_stats_kernel first combines the partials once per
-//         (sequence, head).
+//         partials and forms s[b,j] = sum_h exp(z[b,h,j] - m_bh) / L_bh; with
+//         more than one such CTA per SM hill_attn_stats_kernel first combines
+//         the partials once per (sequence, head).
 //
 // The query rows of a warp's heads are held as mma B fragments in registers
 // for the whole sequence.  Before its dependency wait the kernel builds its
@@ -365,7 +364,7 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
         }
         const int hl = 2 * tig + c;
         if (grp == 0 && hl < gn_of(r))
-          a.partials[((int64_t)cur_b * a.nslot + cur_slot) * H + head0_of(r) + hl] = make_float2(m, l);
+          a.partials[((int64_t)cur_b * H + head0_of(r) + hl) * a.nslot + cur_slot] = make_float2(m, l);
       }
     }
   };
@@ -388,7 +387,7 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
           for (int c = 0; c < kCols; ++c) {
             const int hl = 2 * tig + c;
             if (grp == 0 && hl < gn_of(q))
-              a.partials[((int64_t)b_next * a.nslot + slot) * H + head0_of(q) + hl] = make_float2(-INFINITY, 0.f);
+              a.partials[((int64_t)b_next * H + head0_of(q) + hl) * a.nslot + slot] = make_float2(-INFINITY, 0.f);
           }
         }
       }
@@ -576,74 +575,87 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
 // Combine the per-CTA (max, sum) partials of every head of sequence b, then
 // s[b,j] = sum_h 2^(z2[b,h,j] - m_h) / L_h, one token per thread (logits and
 // partials are in the base-2 scale z2 = z * log2 e, so each term is the
-// softmax weight e^(z - m) / sum e^(z - m)).  Both phases issue all their
-// loads before using them: the partials of a head are spread over 8 threads,
-// and each thread loads the logits of 16 heads of its token at once (they
-// were just written and are mostly L2 resident).
-constexpr int kFinThreads = 256;
-constexpr int kFinChunk = kFinThreads;
-constexpr int kFinPartThreads = 8;                 // threads combining one head
-constexpr int kFinPartMax = 32;                    // partials per thread held in registers
-constexpr int kFinPartFew = 4;                     // the same when a sequence has few (<= 32) slots
+// softmax weight e^(z - m) / sum e^(z - m)).  All loads are issued before any
+// is used: the logits of kFinZ heads of the thread's token (just written and
+// mostly L2 resident), its running importance, and the partials, one head per
+// warp at a time with a partial per lane.
+//
+// Bound by latency (and on long caches by the L2 reads of the logits): between
+// the loads and the store there must be no chain over the heads.  The weights
+// (max, 1/sum) are padded to a multiple of 8 heads whose terms are 0, so that
+// the heads are taken 8 at a time without a branch between them; with a
+// branch per head the 32 terms took 3600-3900 cycles per CTA, which is more
+// than everything else in it (now about 500).  With the partials laid out by
+// head and the heads taken without branches, scores to selection went from
+// 10.4 to 7.1 us on one 4K sequence and from 14.5 to 7.8 on 4 x 16K of one KV
+// head.
+constexpr int kFinThreads = 256;                   // threads (= tokens) of a CTA
+constexpr int kFinHB = 4;                          // heads of a warp whose partials are combined together
+constexpr int kFinU = 5;                           // partials per lane and head held in registers
 constexpr int kHistBins = 2048;                    // leading 11 bits of the order-preserving key
-constexpr int kFinZReg = 32;                       // logits per token held in registers
+constexpr int kFinZ = 32;                          // logits per token held in registers
 constexpr int kFinMaxTpt = 16;                     // token blocks per CTA at most (split step)
 
-// Combine the ns per-CTA partials (max, sum) of every head of sequence b into
-// mh[h] (max) and il[h] (1 / sum): kFinPartThreads threads per head, each
-// holding PM partials in registers with all their loads in flight; slots
-// beyond PM * kFinPartThreads are folded in sequentially.  A warp covers
-// kHeadsPerWarp consecutive heads per pass.  The loop runs while the warp's
-// first head exists, so every lane of a warp takes the same trips and the
-// full-mask shuffles always have all 32 lanes; lanes whose head is past H
-// combine nothing and write nothing.
-template <int PM>
-__device__ __forceinline__ void combine_partials(const FinalizeArgs& a, int b, int ns, float* mh, float* il) {
-  const float2* pb = a.partials + (int64_t)b * a.nslot * a.H;
-  const int sub = threadIdx.x % kFinPartThreads;
-  constexpr int kHeadsPerWarp = 32 / kFinPartThreads;
-  for (int h0 = (threadIdx.x >> 5) * kHeadsPerWarp; h0 < a.H; h0 += kFinThreads / kFinPartThreads) {
-    const int h = h0 + (threadIdx.x & 31) / kFinPartThreads;
-    const bool hv = h < a.H;
-    float2 p[PM];
+__device__ __forceinline__ int pad8(int h) { return (h + 7) & ~7; }
+
+// The (max, 1/sum) of every head of sequence b from its ns per-CTA partials:
+// a warp takes kFinHB of its heads at a time.
+__device__ __forceinline__ void combine_partials(const FinalizeArgs& a, int b, int ns, float2* wt) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int NW = kFinThreads / 32, HB = kFinHB;
+  const float2* pb = a.partials + (int64_t)b * a.H * a.nslot;
+  for (int h0 = warp; h0 < a.H; h0 += NW * HB) {
+    float2 p[HB][kFinU];
 #pragma unroll
-    for (int u = 0; u < PM; ++u) {
-      const int s = sub + u * kFinPartThreads;
-      p[u] = hv && s < ns ? pb[(int64_t)s * a.H + h] : make_float2(-INFINITY, 0.f);
+    for (int i = 0; i < HB; ++i)
+#pragma unroll
+      for (int u = 0; u < kFinU; ++u) {
+        const int h = h0 + NW * i, s = lane + 32 * u;
+        p[i][u] = h < a.H && s < ns ? pb[(int64_t)h * a.nslot + s] : make_float2(-INFINITY, 0.f);
+      }
+    float m[HB], l[HB];
+#pragma unroll
+    for (int i = 0; i < HB; ++i) {
+      m[i] = -INFINITY;
+#pragma unroll
+      for (int u = 0; u < kFinU; ++u) m[i] = fmaxf(m[i], p[i][u].x);
+      l[i] = 0.f;
+#pragma unroll
+      for (int u = 0; u < kFinU; ++u) l[i] += p[i][u].y > 0.f ? p[i][u].y * ex2(p[i][u].x - m[i]) : 0.f;
     }
-    float m = -INFINITY;
+    // slots past 32 * kFinU (the dealing kernel's): a running maximum
+    for (int s0 = 32 * kFinU; s0 < ns; s0 += 32) {
 #pragma unroll
-    for (int u = 0; u < PM; ++u) m = fmaxf(m, p[u].x);
-    for (int s = sub + PM * kFinPartThreads; hv && s < ns; s += kFinPartThreads)
-      m = fmaxf(m, pb[(int64_t)s * a.H + h].x);
-#pragma unroll
-    for (int o = kFinPartThreads / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    float l = 0.f;
-#pragma unroll
-    for (int u = 0; u < PM; ++u) l += p[u].y > 0.f ? p[u].y * ex2(p[u].x - m) : 0.f;
-    for (int s = sub + PM * kFinPartThreads; hv && s < ns; s += kFinPartThreads) {
-      const float2 q = pb[(int64_t)s * a.H + h];
-      l += q.y > 0.f ? q.y * ex2(q.x - m) : 0.f;
+      for (int i = 0; i < HB; ++i) {
+        const int h = h0 + NW * i, s = s0 + lane;
+        const float2 q = h < a.H && s < ns ? pb[(int64_t)h * a.nslot + s] : make_float2(-INFINITY, 0.f);
+        if (!(q.y > 0.f)) continue;
+        const float mn = fmaxf(m[i], q.x);
+        l[i] = (l[i] > 0.f ? l[i] * ex2(m[i] - mn) : 0.f) + q.y * ex2(q.x - mn);
+        m[i] = mn;
+      }
     }
+    float mw[HB];
 #pragma unroll
-    for (int o = kFinPartThreads / 2; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if (sub == 0 && hv) {
-      mh[h] = m;
-      il[h] = 1.f / l;
-    }
+    for (int i = 0; i < HB; ++i) mw[i] = warp_max(m[i]);
+#pragma unroll
+    for (int i = 0; i < HB; ++i) l[i] = warp_sum(l[i] > 0.f ? l[i] * ex2(m[i] - mw[i]) : 0.f);
+#pragma unroll
+    for (int i = 0; i < HB; ++i)
+      if (lane == 0 && h0 + NW * i < a.H) wt[h0 + NW * i] = make_float2(mw[i], 1.f / l[i]);
   }
 }
 
 // STATS: the per-head (max, 1/sum) come from hill_attn_stats_kernel instead of
-// every CTA combining the partials itself (long sequences: many CTAs).  KVH:
-// per-KV-head importance (a.kvh), a variant of its own so that its group sums
-// do not weigh on the registers of the plain kernel.
+// every CTA combining the partials itself.  KVH: per-KV-head importance
+// (a.kvh), a variant of its own so that its group sums do not weigh on the
+// registers of the plain kernel.
 template <bool STATS, bool KVH>
-__global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize_kernel(FinalizeArgs a) {
-  extern __shared__ float fsm[];
-  float* mh = fsm;            // [H]
-  float* il = fsm + a.H;      // [H]
-  uint32_t* hcount = reinterpret_cast<uint32_t*>(fsm + 2 * a.H);   // [kHistBins] when a.hist0
+__global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize_kernel(const FinalizeArgs a) {
+  extern __shared__ __align__(16) float fsm[];
+  const int hp = pad8(a.H);
+  float2* wt = reinterpret_cast<float2*>(fsm);                     // [hp] (max, 1/sum)
+  uint32_t* hcount = reinterpret_cast<uint32_t*>(fsm + 2 * hp);    // [kHistBins] when a.hist0
   // The lengths are inputs of the call: this kernel only ever follows the
   // scoring kernel of the same call, whose own dependency wait covered every
   // earlier write, so they are read before this kernel's wait and overlap
@@ -652,13 +664,16 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
   const int b = blockIdx.y;
   int len = a.lens[b];
   len = len < 0 ? 0 : (len > a.cap ? a.cap : len);
-  // this CTA's tokens: a.tpt blocks of kFinChunk from jb
-  const int jb = blockIdx.x * kFinChunk * a.tpt;
+  // this CTA's tokens: a.tpt blocks of kFinThreads from jb
+  const int jb = blockIdx.x * kFinThreads * a.tpt;
   if (jb >= len) return;
   // the scoring CTAs that met b wrote slots 0 .. ns-1
   // (every thread counts the tiles of a share of the sequences)
   __shared__ int s_first, s_total;
   if (threadIdx.x == 0) s_first = s_total = 0;
+  if (threadIdx.x < hp - a.H) wt[a.H + threadIdx.x] = make_float2(-kNegHuge, 0.f);   // 0 * 2^(z - huge) = 0
+  if (a.hist0)
+    for (int i = threadIdx.x; i < kHistBins; i += kFinThreads) hcount[i] = 0u;
   __syncthreads();
   {
     int f = 0, t = 0;
@@ -680,108 +695,99 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
   const int ns = ((first_item + items - 1) / per - first_item / per + 1) * a.spc;
   pdl_wait();
   pdl_launch_dependents();
-  // this token's logits of the first kFinZReg heads, loaded before the
-  // partials are combined so that both round trips overlap
+  // This token's logits of heads [h0, h0 + kFinZ), 8 at a time (those past H
+  // repeat the last head, with weight 0).  Threads past the length read the
+  // last token's and write nothing.
   int j = jb + threadIdx.x;
-  bool valid = j < len;
-  const float* zp = a.logits + (int64_t)b * a.H * a.lstride + j;
-  float zr[kFinZReg];
+  const float* zb = a.logits + (int64_t)b * a.H * a.lstride;
+  float zr[kFinZ];
+  auto load_z = [&](int h0) {
+    const float* zp = zb + min(j, len - 1);
 #pragma unroll
-  for (int u = 0; u < kFinZReg; ++u) zr[u] = (valid && u < a.H) ? zp[(int64_t)u * a.lstride] : 0.f;
+    for (int u0 = 0; u0 < kFinZ; u0 += 8)
+      if (h0 + u0 < a.H) {
+#pragma unroll
+        for (int u = u0; u < u0 + 8; ++u) zr[u] = zp[(int64_t)min(h0 + u, a.H - 1) * a.lstride];
+      }
+  };
+  float acc = 0.f;   // the running importance of this token
+  auto load_acc = [&]() {
+    if (!KVH && a.accum) acc = a.accum[(int64_t)b * a.cap + min(j, len - 1)];
+  };
+  load_z(0);
+  load_acc();
   if constexpr (STATS) {
-    for (int h = threadIdx.x; h < a.H; h += kFinThreads) {
-      const float2 st = a.stats[(int64_t)b * a.H + h];
-      mh[h] = st.x;
-      il[h] = st.y;
-    }
+    for (int h = threadIdx.x; h < a.H; h += kFinThreads) wt[h] = a.stats[(int64_t)b * a.H + h];
+  } else {
+    combine_partials(a, b, ns, wt);
   }
-  if constexpr (!STATS) {
-    // ns is the same for the whole CTA, so every warp takes the same branch
-    if (ns <= kFinPartThreads * kFinPartFew) combine_partials<kFinPartFew>(a, b, ns, mh, il);
-    else combine_partials<kFinPartMax>(a, b, ns, mh, il);
-  }
-  if (a.hist0)
-    for (int i = threadIdx.x; i < kHistBins; i += kFinThreads) hcount[i] = 0u;
   __syncthreads();
   for (int blk = 0;;) {   // the CTA's token blocks (one unless a.tpt > 1)
-  if (KVH && valid) {
-    // per-KV-head importance: the sum over each group of G query heads,
-    // stored as soon as the group is complete (heads of a group are adjacent)
-    const int G = a.H / a.Hkv;
-    int g = 0, in_g = 0;   // the group being summed and its heads so far
-    auto put = [&](float v) {
-      const int64_t o = ((int64_t)b * a.Hkv + g) * a.cap + j;
-      if (a.scores) a.scores[o] = v;
-      if (a.accum) a.accum[o] += v;
-    };
-    float sg = 0.f;
+    const bool valid = j < len;
+    float s = 0.f;
+    int g = 0, in_g = 0;   // KVH: the group being summed and its heads so far
+    const int G = KVH ? a.H / a.Hkv : 1;
+    for (int h0 = 0;;) {
 #pragma unroll
-    for (int u = 0; u < kFinZReg; ++u)
-      if (u < a.H) {
-        sg += ex2(zr[u] - mh[u]) * il[u];
-        if (++in_g == G) {
-          put(sg);
-          ++g;
-          in_g = 0;
-          sg = 0.f;
-        }
-      }
-    for (int h = kFinZReg; h < a.H; h += 16) {
-      float z[16];
+      for (int u0 = 0; u0 < kFinZ; u0 += 8)
+        if (h0 + u0 < a.H) {
+          float t[8], w[8];
 #pragma unroll
-      for (int u = 0; u < 16; ++u) z[u] = h + u < a.H ? zp[(int64_t)(h + u) * a.lstride] : 0.f;
+          for (int u = 0; u < 8; u += 2) {
+            const float4 x = *reinterpret_cast<const float4*>(wt + h0 + u0 + u);   // two heads
+            t[u] = ex2(zr[u0 + u] - x.x), w[u] = x.y;
+            t[u + 1] = ex2(zr[u0 + u + 1] - x.z), w[u + 1] = x.w;
+          }
+          if constexpr (KVH) {
+            // the sum over each group of G query heads, stored as soon as the
+            // group is complete (heads of a group are adjacent)
 #pragma unroll
-      for (int u = 0; u < 16; ++u)
-        if (h + u < a.H) {
-          sg += ex2(z[u] - mh[h + u]) * il[h + u];
-          if (++in_g == G) {
-            put(sg);
-            ++g;
-            in_g = 0;
-            sg = 0.f;
+            for (int u = 0; u < 8; ++u) {
+              s = __fmaf_rn(t[u], w[u], s);
+              if (++in_g == G && h0 + u0 + u < a.H) {
+                if (valid) {
+                  const int64_t o = ((int64_t)b * a.Hkv + g) * a.cap + j;
+                  if (a.scores) a.scores[o] = s;
+                  if (a.accum) a.accum[o] += s;
+                }
+                ++g;
+                in_g = 0;
+                s = 0.f;
+              }
+            }
+          } else {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s = __fmaf_rn(t[u], w[u], s);
           }
         }
+      h0 += kFinZ;
+      if (h0 >= a.H) break;
+      load_z(h0);
     }
-  } else if (!KVH && valid) {
-    float s = 0.f;
-#pragma unroll
-    for (int u = 0; u < kFinZReg; ++u)
-      if (u < a.H) s += ex2(zr[u] - mh[u]) * il[u];
-    int h = kFinZReg;
-    for (; h + 16 <= a.H; h += 16) {
-      float z[16];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) z[u] = zp[(int64_t)(h + u) * a.lstride];
-#pragma unroll
-      for (int u = 0; u < 16; ++u) s += ex2(z[u] - mh[h + u]) * il[h + u];
+    if (!KVH && valid) {
+      const int64_t o = (int64_t)b * a.cap + j;
+      if (a.scores) a.scores[o] = s;
+      float key = s;
+      if (a.accum) {
+        key = acc + s;
+        a.accum[o] = key;
+      }
+      if (a.hist0 && j < len - min(a.recent, len)) atomicAdd(&hcount[ordered_key(key) >> 21], 1u);
     }
-    for (; h < a.H; ++h) s += ex2(zp[(int64_t)h * a.lstride] - mh[h]) * il[h];
-    const int64_t o = (int64_t)b * a.cap + j;
-    if (a.scores) a.scores[o] = s;
-    float key = s;
-    if (a.accum) {
-      key = a.accum[o] + s;
-      a.accum[o] = key;
-    }
-    if (a.hist0 && j < len - min(a.recent, len)) atomicAdd(&hcount[ordered_key(key) >> 21], 1u);
-  }
-  // The logits are dead once read: drop this warp's lines from L2 without
-  // writing them back (each 128-byte line holds the warp's 32 tokens of one
-  // head; every lane has consumed its loads before the warp passes the sync).
-  {
-    const int j0 = j - (int)(threadIdx.x & 31);
+    // The logits are dead once read: drop this warp's lines from L2 without
+    // writing them back (each 128-byte line holds the warp's 32 tokens of one
+    // head; every lane has consumed its loads before the warp passes the sync).
+    // A warp wholly past the length has read the last token's lines, which
+    // belong to another warp.
+    const int jw = j - (int)(threadIdx.x & 31);
     __syncwarp();
-    if (j0 < len)
-      for (int h = threadIdx.x & 31; h < a.H; h += 32)
-        l2_discard_line(a.logits + ((int64_t)b * a.H + h) * a.lstride + j0);
-  }
-  // the next block of tokens (its logits loaded before they are used)
-  if (++blk >= a.tpt || jb + blk * kFinChunk >= len) break;
-  j = jb + blk * kFinChunk + threadIdx.x;
-  valid = j < len;
-  zp = a.logits + (int64_t)b * a.H * a.lstride + j;
-#pragma unroll
-  for (int u = 0; u < kFinZReg; ++u) zr[u] = (valid && u < a.H) ? zp[(int64_t)u * a.lstride] : 0.f;
+    if (jw < len)
+      for (int h = threadIdx.x & 31; h < a.H; h += 32) l2_discard_line(zb + (int64_t)h * a.lstride + jw);
+    // the next block of tokens
+    if (++blk >= a.tpt || jb + blk * kFinThreads >= len) break;
+    j = jb + blk * kFinThreads + threadIdx.x;
+    load_z(0);
+    load_acc();
   }
   if (a.hist0) {
     __syncthreads();
@@ -805,7 +811,7 @@ __global__ void __launch_bounds__(kStatsWarps * 32) hill_attn_stats_kernel(Final
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int pair = blockIdx.x * kStatsWarps + warp;
   if (pair >= a.B * a.H) return;
-  const int b = pair / a.H, h = pair - b * a.H;
+  const int b = pair / a.H;
   // the slots 0 .. ns-1 of b (lengths are inputs of the call: read before the wait)
   int f = 0, t = 0;
   for (int bb = lane; bb < a.B; bb += 32) {
@@ -828,14 +834,14 @@ __global__ void __launch_bounds__(kStatsWarps * 32) hill_attn_stats_kernel(Final
   const int ns = items == 0 ? 0 : ((f + items - 1) / per - f / per + 1) * a.spc;
   pdl_wait();
   pdl_launch_dependents();
-  const float2* pb = a.partials + (int64_t)b * a.nslot * a.H + h;
+  const float2* pb = a.partials + (int64_t)pair * a.nslot;
   float m = -INFINITY, l = 0.f;
   for (int s0 = lane; s0 < ns; s0 += 32 * kStatsPer) {
     float2 p[kStatsPer];
 #pragma unroll
     for (int u = 0; u < kStatsPer; ++u) {
       const int s = s0 + 32 * u;
-      p[u] = s < ns ? pb[(int64_t)s * a.H] : make_float2(-INFINITY, 0.f);
+      p[u] = s < ns ? pb[s] : make_float2(-INFINITY, 0.f);
     }
 #pragma unroll
     for (int u = 0; u < kStatsPer; ++u) {
@@ -908,6 +914,14 @@ cudaError_t launch_score(const ScoreArgs& a, int dtype, int G, bool raw, bool f8
   return f8 ? launch_score_m<1, true>(a, G, raw, deal, grid, st) : launch_score_m<1, false>(a, G, raw, deal, grid, st);
 }
 
+template <bool STATS>
+static cudaError_t launch_finalize_t(const FinalizeArgs& a, cudaStream_t st) {
+  const dim3 grid((a.cap + kFinThreads * a.tpt - 1) / (kFinThreads * a.tpt), a.B);
+  const size_t smem = (size_t)((a.H + 7) & ~7) * sizeof(float2) + (a.hist0 ? kHistBins * sizeof(uint32_t) : 0);
+  return a.kvh ? launch_pdl(hill_attn_finalize_kernel<STATS, true>, grid, dim3(kFinThreads), smem, st, 0, a)
+               : launch_pdl(hill_attn_finalize_kernel<STATS, false>, grid, dim3(kFinThreads), smem, st, 0, a);
+}
+
 cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t st, int* kernels,
                                  bool two_kernel) {
   FinalizeArgs a = a0;
@@ -918,24 +932,22 @@ cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t s
   // CTAs instead of trickling through in many.
   if (two_kernel)
     while (a.tpt < kFinMaxTpt &&
-           (long long)a.B * ((a.cap + kFinChunk * a.tpt - 1) / (kFinChunk * a.tpt)) > 2LL * sms)
+           (long long)a.B * ((a.cap + kFinThreads * a.tpt - 1) / (kFinThreads * a.tpt)) > 2LL * sms)
       a.tpt <<= 1;
-  dim3 grid((a.cap + kFinChunk * a.tpt - 1) / (kFinChunk * a.tpt), a.B);
-  const size_t smem = 2 * a.H * sizeof(float) + (a.hist0 ? kHistBins * sizeof(uint32_t) : 0);
-  // more than two normalisation CTAs per SM: combine the partials once per
-  // (b, h) in a kernel of their own instead of once per CTA
-  if (a.stats && (two_kernel || (long long)grid.x * grid.y > 2LL * sms)) {
+  // With more than one CTA per SM the partials are combined once per (b, h)
+  // in a kernel of their own instead of once per CTA: scores to selection at
+  // 4 x 16K tokens of one KV head (304 partials per head) 23.8 against 27.7
+  // us, 4 x 16-32K 142.1 against 142.6, 1 x 128K the same; up to one CTA per
+  // SM the second launch costs more than it saves (about 2 us).
+  if (two_kernel || (long long)a.B * ((a.cap + kFinThreads - 1) / kFinThreads) > sms) {
     *kernels = 2;
     const int pairs = a.B * a.H;
     cudaError_t e = launch_pdl(hill_attn_stats_kernel, dim3((pairs + kStatsWarps - 1) / kStatsWarps),
                                dim3(kStatsWarps * 32), 0, st, 0, a);
-    if (e != cudaSuccess) return e;
-    return a.kvh ? launch_pdl(hill_attn_finalize_kernel<true, true>, grid, dim3(kFinThreads), smem, st, 0, a)
-                 : launch_pdl(hill_attn_finalize_kernel<true, false>, grid, dim3(kFinThreads), smem, st, 0, a);
+    return e != cudaSuccess ? e : launch_finalize_t<true>(a, st);
   }
   *kernels = 1;
-  return a.kvh ? launch_pdl(hill_attn_finalize_kernel<false, true>, grid, dim3(kFinThreads), smem, st, 0, a)
-               : launch_pdl(hill_attn_finalize_kernel<false, false>, grid, dim3(kFinThreads), smem, st, 0, a);
+  return launch_finalize_t<false>(a, st);
 }
 
 }  // namespace hill

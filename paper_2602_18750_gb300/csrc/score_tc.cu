@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) hill_score_tc_kernel(const __gr
           }
         const float mw = warp_max(m);
         const float lw = warp_sum(l > 0.f ? l * ex2(m - mw) : 0.f);
-        if (lane == 0) a.partials[((int64_t)bb * a.nslot + slot) * H + h] = make_float2(mw, lw);
+        if (lane == 0) a.partials[((int64_t)bb * H + h) * a.nslot + slot] = make_float2(mw, lw);
       }
       const bool ok = epi_meet(base_addr + kOffBarEpi + 8);
       epi_ph ^= 1u;

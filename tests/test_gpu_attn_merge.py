@@ -1,0 +1,74 @@
+"""The sparse attention's split of the selected rows over warps and CTAs and the merges that follow, against float64:
+pairs (sequence, KV head) held by one warp, by several warps of a CTA and by many CTAs, groups served in passes of 16
+heads, empty sequences, and a workspace that holds arbitrary data before the call.
+"""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from parity_util import check_attn
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def H():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_18750_gb300 import build, hill
+    build.build()
+    hill.load()
+    return hill
+
+
+# (B, H, Hkv, tokens, kept per sequence)
+CASES = [
+    (1, 1, 1, 4096, [1]),                    # one batch: one warp
+    (1, 2, 2, 4096, [33]),                   # two batches per pair
+    (1, 1, 1, 40000, [40000]),               # one pair over all CTAs (1250 batches, two per warp)
+    (1, 32, 1, 20000, [19999]),              # two passes of 16 heads, each over half of the CTAs
+    (2, 20, 1, 4096, [4000, 0]),             # passes of 16 and 4 heads, an empty sequence
+    (3, 40, 1, 2048, [2048, 31, 32]),        # passes of 16, 16 and 8
+    (2, 24, 8, 4096, [3000, 257]),           # groups of 3
+    (4, 32, 32, 4096, [819, 0, 1, 300]),     # many short pairs
+    (8, 32, 32, 2048, [1999, 7, 0, 1024, 33, 64, 65, 2048]),
+    (5, 14, 2, 5000, [5000, 4999, 1, 0, 2500]),   # groups of 7
+]
+
+
+@pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"B{c[0]}H{c[1]}kv{c[2]}n{max(c[4])}")
+def test_attention_over_every_split(H, case, dtype):
+    B, Hq, Hkv, n, kept = case
+    g = torch.Generator(device="cuda").manual_seed(n + Hq)
+    K, V = (torch.randn(B, Hkv, n, 128, generator=g, device="cuda").to(dtype) for _ in range(2))
+    q = torch.randn(B, Hq, 128, generator=g, device="cuda").to(dtype)
+    desc = H.make_desc(q, K, V)
+    max_k = max(kept)
+    idx = torch.full((B, max_k), -1, dtype=torch.int32, device="cuda")
+    sets = []
+    for b, m in enumerate(kept):
+        t = torch.randperm(n, generator=g, device="cuda")[:m].sort().values
+        idx[b, :m] = t.int()
+        sets.append(t)
+    count = torch.tensor(kept, dtype=torch.int32, device="cuda")
+    out = torch.full((B, Hq, 128), float("nan"), device="cuda")
+    ws = H.alloc_workspace(desc, 0, max_k)
+    ws.fill_(0xFF)
+    ref = np.zeros((B, Hq, 128))
+    G = Hq // Hkv
+    for b, t in enumerate(sets):
+        for h in range(Hq if len(t) else 0):
+            z = K[b, h // G, t].double() @ q[b, h].double() / math.sqrt(128)
+            ref[b, h] = (torch.softmax(z, 0) @ V[b, h // G, t].double()).cpu().numpy()
+    first = None
+    for _ in range(2):   # (the second call finds what the first one left in the workspace)
+        H.hill_gather_sparse_attn(desc, q, K, V, idx, count, max_k, out, ws)
+        H.hill_sync_status()
+        check_attn(out.cpu().numpy(), ref)
+        if first is not None:
+            assert torch.equal(out, first), "the merge order must not depend on which CTA arrives last"
+        first = out.clone()
+        out.fill_(float("nan"))

@@ -1,0 +1,55 @@
+"""The normalisation of the ATTN importance against float64: head counts that are not a multiple of the 8 taken at a
+time or exceed the 32 held at a time, many partials per head (several warps per KV head), one and two kernels, ragged
+and empty sequences; with the running importance and the selection that is fed by its digit counts.
+"""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+# (B, H, Hkv, tokens of each sequence)
+CASES = [
+    (1, 1, 1, [1]),
+    (2, 9, 3, [257, 0]),
+    (1, 32, 1, [6000]),              # 1216 partials per head, combined in the one kernel
+    (3, 8, 1, [30000, 16000, 1]),    # the same in two kernels
+    (2, 28, 4, [3001, 2999]),
+    (2, 64, 8, [9000, 4097]),        # two rounds of 32 heads
+    (1, 72, 8, [70001]),             # three, in two kernels
+    (5, 40, 40, [700, 31, 32, 33, 640]),
+]
+
+
+@pytest.mark.parametrize("case", CASES, ids=lambda c: f"B{c[0]}H{c[1]}kv{c[2]}n{max(c[3])}")
+def test_scores_and_selection(case):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_18750_gb300 import build, hill as H
+    build.build()
+    B, Hq, Hkv, lens = case
+    n, G = max(lens), Hq // Hkv
+    g = torch.Generator(device="cuda").manual_seed(n + Hq)
+    K = torch.randn(B, Hkv, n, 128, generator=g, device="cuda").half()
+    q = (3 * torch.randn(B, Hq, 128, generator=g, device="cuda")).half()
+    accum = torch.rand(B, n, generator=g, device="cuda") * Hq / n
+    before = accum.double()
+    desc = H.make_desc(q, K)
+    kept = [max(1, m // 5) if m else 0 for m in lens]
+    dev = lambda v: torch.tensor(v, dtype=torch.int32, device="cuda")  # noqa: E731
+    scores = torch.zeros(B, n, device="cuda")
+    idx = torch.zeros(B, max(kept), dtype=torch.int32, device="cuda")
+    count = torch.zeros(B, dtype=torch.int32, device="cuda")
+    ws = H.alloc_workspace(desc, 0, max(kept))
+    H.hill_evict_step(desc, q, K, None, dev(lens), dev(kept), max(kept), 0, accum, scores, idx, count, None, ws)
+    H.hill_sync_status()
+    assert count.tolist() == kept
+    for b, m in enumerate(lens):
+        z = torch.stack([K[b, h // G, :m].double() @ q[b, h].double() for h in range(Hq)]) / np.sqrt(128)
+        ref = torch.softmax(z, -1).sum(0)
+        # 32-bit logits of magnitude up to ~15: a few 2^-24 of them in the exponent, and as much in the sums
+        assert torch.all((scores[b, :m].double() - ref).abs() <= 2e-5 * ref.clamp_min(1e-30)) or m == 0
+        assert torch.all((accum[b, :m].double() - before[b, :m] - scores[b, :m].double()).abs() <= 1e-6)
+        # the selection is exact on the kernel's own sums
+        order = torch.sort(accum[b, :m], descending=True, stable=True).indices[:kept[b]]
+        assert torch.equal(idx[b, :kept[b]].long(), order.sort().values)
