@@ -497,6 +497,10 @@ hill_status run_attn(const hill_desc* d, const void* q, const void* k, const voi
   // selected rows, then one merge of the split partials over all heads
   const int G = d->num_q_heads / d->num_kv_heads;
   a.Gs = G;
+  bool done = false;
+  const hill_status cs = from_cuda(launch_sparse_attn_clusters(a, d->dtype, di.sms, st, &done));
+  if (done && cs == HILL_OK) counted(cudaSuccess, 1);
+  if (done || cs != HILL_OK) return cs;
   return head_passes(d, false, [&](int, int, int hoff, int Gn, bool) {
     a.hoff = hoff;
     a.Gn = Gn;

@@ -32,9 +32,25 @@
 // groups run in passes of 16.  When a warp's segment holds
 // all batches of a (b, g) it writes the output; otherwise it writes a partial
 // (max, sum, o) that hill_attn_combine_kernel merges.
+//
+// Small calls are bound by latency, and there the merge is the longest part: a
+// second launch, its reads of the counts and of the partials.  With few
+// (b, g, pass) triples a cluster of CTAs takes each (CL): its warps share the
+// triple's batches, the CTAs merge their warps' partials in shared memory and
+// push them to one of them, which writes the output.  Such a CTA knows its
+// triple from the start, so the queries are loaded before the dependency wait
+// and the first index entries together with the count.  Measured: one 4K sequence of
+// 32 heads (k = 819) 7.5 -> 5.0 us, 1 x 128K with 8 KV heads (k = 2048) 8.8 ->
+// 6.7, 4 x 16K of one KV head (two passes over 32 heads) 18.3 -> 7.9.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "hill_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace hill {
 namespace {
@@ -49,8 +65,17 @@ constexpr int kHalfBytes = kBatch * 128;             // 32 rows x 64 dims, swizz
 struct AttnCfg {
   // K dims 0-63 | K dims 64-127 | V dims 0-63 | V dims 64-127
   static constexpr int kSlotBytes = 4 * kHalfBytes;
-  static constexpr int kSmem = kAW * kSlotBytes + 128;   // + alignment slack
+  static constexpr int smem(int warps) { return warps * kSlotBytes + 128; }   // + alignment slack
 };
+
+constexpr int kPS = 2 + kHeadDim;   // one partial of a head: max, sum, o[kHeadDim]
+constexpr int kMaxAttnCluster = 8;
+
+// CL: partials of this CTA's share of the triple's heads, from every CTA of the cluster
+template <int G>
+constexpr int recv_floats() {
+  return (G + kMaxAttnCluster - 1) * kPS;
+}
 
 // Position of a batch in the list: table unit u (a sequence b, or with
 // per-KV-head selection a pair (b, g)), sequence, KV head, batch within (b, g).
@@ -71,25 +96,73 @@ __device__ __forceinline__ void warp_segment(int total, int nwarps, int w, int& 
   t1 = min(total, t0 + per);
 }
 
-template <int DT, int G>
-__global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __grid_constant__ AttnArgs a) {
+template <int DT, int G, bool CL, int NW>
+__global__ void __launch_bounds__(NW * 32, kAW / NW) hill_sparse_attn_kernel(const __grid_constant__ AttnArgs a) {
   extern __shared__ unsigned char asmem[];
-  __shared__ int s_bstart[kMaxBatchAttn + 1];
-  __shared__ int s_nbat[kMaxBatchAttn];
-  __shared__ int s_cnt[kMaxBatchAttn];
+  __shared__ int s_bstart[CL ? 1 : kMaxBatchAttn + 1];
+  __shared__ int s_nbat[CL ? 1 : kMaxBatchAttn];
+  __shared__ int s_cnt[CL ? 1 : kMaxBatchAttn];
+  __shared__ float s_recv[CL ? recv_floats<G>() : 1];
+  __shared__ int s_has[NW];   // CL: the warp has a partial
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = lane >> 2, tig = lane & 3;
+  constexpr int kRB = G > 8 ? 2 : 1;          // row blocks of 8 heads
+  // CL: the cluster's triple (b, g, pass), its table unit and its heads
+  int C = 1, rank = 0, tu = 0, tb = 0, tg = 0;
+  int Gn = G <= 2 ? G : a.Gn, hoff = a.hoff;
+  if constexpr (CL) {
+    C = (int)cg::this_cluster().num_blocks();
+    rank = (int)cg::this_cluster().block_rank();
+    if (C > 1) cg::this_cluster().barrier_arrive();   // every CTA has started (waited for before the first push)
+    const int P = (a.Gs + 15) / 16, triple = blockIdx.x / C, bg = triple / P;
+    hoff = 16 * (triple - bg * P);
+    Gn = min(16, a.Gs - hoff);
+    tb = bg / a.Hkv;
+    tg = bg - tb * a.Hkv;
+    tu = a.kvh ? bg : tb;
+  }
+  uint32_t qa[kRB][8][2];                     // q rows of the group as A fragments
+  bool head_ok[kRB];
+#pragma unroll
+  for (int rb = 0; rb < kRB; ++rb) head_ok[rb] = grp + 8 * rb < Gn;
+  auto load_q = [&](int b, int g) {
+    const auto* q32 = static_cast<const uint32_t*>(a.q);
+#pragma unroll
+    for (int rb = 0; rb < kRB; ++rb) {
+      const bool ok = head_ok[rb];
+      const int64_t row = ok ? ((int64_t)b * a.q_sb + (int64_t)(g * a.Gs + hoff + 8 * rb + grp) * a.q_sh) / 2 : 0;
+#pragma unroll
+      for (int kb = 0; kb < 8; ++kb) {
+        qa[rb][kb][0] = ok ? __ldg(q32 + row + kb * 8 + tig) : 0u;
+        qa[rb][kb][1] = ok ? __ldg(q32 + row + kb * 8 + 4 + tig) : 0u;
+      }
+    }
+  };
+  if constexpr (CL) load_q(tb, tg);   // (an input of the call: include/hill.h)
   pdl_wait();
   // No early trigger (here and in the combine): the attention runs beside
   // the K stream of later layers, and a dependent launched early would hold
   // SMs idle while it waits (measured: the pipelined step is 2 % faster).
 
+  // CL: this cluster's count, and the index entries of warp w's first batch if
+  // every warp has one at most
+  int n_unit = 0, nb_unit = 0, j_first = -1;
+  if constexpr (CL) {
+    const int e = (rank * NW + warp) * kBatch + lane;
+    if (e < a.max_k) j_first = a.idx[(int64_t)tu * a.max_k + e];
+    n_unit = clamp_count(a, tu);
+    nb_unit = (n_unit + kBatch - 1) / kBatch;
+  }
+  auto cnt_of = [&](int u) { return CL ? n_unit : s_cnt[u]; };
+  auto nbat_of = [&](int u) { return CL ? nb_unit : s_nbat[u]; };
   // table units: sequences (every KV head reads the same set, Hkv * nbat
   // batches per unit, ordered g, bi), or with per-KV-head selection the pairs
   // (b, g) (nbat batches per unit)
   const int R = a.kvh ? a.B * a.Hkv : a.B;
   const int upb = a.kvh ? 1 : a.Hkv;   // KV heads per unit
-  for (int u = threadIdx.x; u < R; u += kAThreads) {
+  if constexpr (!CL) {
+  for (int u = threadIdx.x; u < R; u += (NW * 32)) {
     const int n = clamp_count(a, u);
     s_cnt[u] = n;
     s_nbat[u] = (n + kBatch - 1) / kBatch;
@@ -104,12 +177,13 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
     s_bstart[R] = acc;
   }
   __syncthreads();
-  const int total = s_bstart[R];
-  const int nwarps = gridDim.x * kAW;
-  const int gw = blockIdx.x * kAW + warp;
+  }
+  const int total = CL ? nb_unit : s_bstart[R];
+  const int nwarps = (CL ? C : gridDim.x) * NW;
+  const int gw = (CL ? rank : blockIdx.x) * NW + warp;
   int t0, t1;
   warp_segment(total, nwarps, gw, t0, t1);
-  if (t0 >= t1) return;
+  if (!CL && t0 >= t1) return;
 
   // 128-byte aligned slots: every swizzled row is one bank-aligned line
   const uint32_t slot0 = ((smem_addr(asmem) + 127u) & ~127u) + warp * AttnCfg::kSlotBytes;
@@ -120,7 +194,9 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
 
   // position of batch t0 (binary search once), then advanced one batch at a time
   Pos first;
-  {
+  if constexpr (CL) {
+    first = Pos{tu, tb, tg, t0};
+  } else {
     int lo = 0, hi = R;
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
@@ -139,6 +215,10 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
     }
   }
   auto advance = [&](Pos& p) {
+    if constexpr (CL) {
+      ++p.bi;
+      return;
+    }
     if (p.u >= R) return;
     if (++p.bi < s_nbat[p.u]) return;
     p.bi = 0;
@@ -155,12 +235,12 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
   // until the batch is issued one iteration later, where it is checked.
   auto load_idx = [&](const Pos& p) -> int {
     const int e = p.bi * kBatch + lane;
-    return e < s_cnt[p.u] ? a.idx[(int64_t)p.u * a.max_k + e] : -1;
+    return e < cnt_of(p.u) ? a.idx[(int64_t)p.u * a.max_k + e] : -1;
   };
   // An entry of the batch at p that lies outside [0, cap) is reported and
   // skipped (-1: no token).
   auto check = [&](const Pos& p, int jj) -> int {
-    if (p.bi * kBatch + lane < s_cnt[p.u] && (jj < 0 || jj >= a.cap)) {
+    if (p.bi * kBatch + lane < cnt_of(p.u) && (jj < 0 || jj >= a.cap)) {
       raise_error(a.err, kErrDevArg);
       jj = -1;
     }
@@ -197,14 +277,20 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
   // cp.async groups complete in the order K(t), V(t), K(t + 1), V(t + 1), ...
   // The index entries of batch t + 2 are loaded when K(t + 1) is issued.
   Pos pc = first, pi = first, pl = first;
-  int jcur = check(pi, load_idx(pl));           // entries of the batch being issued
+  unsigned vm_cur = 0u, vm_next = 0u;
+  int jcur = -1, jnext = -1;                    // entries of the batch being issued, and of the next
+  if (!CL || t0 < t1) {
+  // (CL, one batch per warp: its entries are here already)
+  const bool have = CL && t0 == gw;
+  jcur = check(pi, !have ? load_idx(pl) : (pl.bi * kBatch + lane < cnt_of(pl.u) ? j_first : -1));
   advance(pl);
-  unsigned vm_cur = __ballot_sync(0xffffffffu, jcur >= 0), vm_next = 0u;
+  vm_cur = __ballot_sync(0xffffffffu, jcur >= 0);
   issue_rows(pi, sk, kbase, a.k_sb, a.k_sh, ksn, jcur);
   issue_rows(pi, sv, vbase, a.v_sb, a.v_sh, vsn, jcur);
   advance(pi);
-  int jnext = t0 + 1 < t1 ? load_idx(pl) : -1;
+  jnext = t0 + 1 < t1 ? load_idx(pl) : -1;
   advance(pl);
+  }
 
   // mma.sync fragments: grp = lane/4, tig = lane%4.  S accumulators: row grp
   // (+8 with 16 heads: row block rb = 1) = query head grp (+8) of the group
@@ -212,21 +298,13 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
   // group has fewer heads than the power-of-two template), columns = tokens
   // nb*8 + 2*tig + {0,1}.  O^T accumulators, one set per row block: rows =
   // dims db*16 + grp (+8), columns = heads 8*rb + 2*tig, 8*rb + 2*tig + 1.
-  constexpr int kRB = G > 8 ? 2 : 1;          // row blocks of 8 heads
-  const int grp = lane >> 2, tig = lane & 3;
-  const int Gn = G <= 2 ? G : a.Gn;
-  bool head_ok[kRB];
-#pragma unroll
-  for (int rb = 0; rb < kRB; ++rb) head_ok[rb] = grp + 8 * rb < Gn;
   const int hA = 2 * tig, hB = 2 * tig + 1;   // heads of this lane's O^T columns (in a row block)
   float m_run[kRB], l_run[kRB];               // softmax state of head grp + 8*rb (base 2)
   float oacc[kRB][8][4];
-  uint32_t qa[kRB][8][2];                     // q rows of the group as A fragments
   int cb = -1, cg = -1, cu = -1;              // the (b, g) being accumulated and its unit
   const int per = (total + nwarps - 1) / nwarps;
 
   auto reset = [&](int b, int g) {
-    const auto* q32 = static_cast<const uint32_t*>(a.q);
 #pragma unroll
     for (int rb = 0; rb < kRB; ++rb) {
       m_run[rb] = -INFINITY;
@@ -235,23 +313,17 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
       for (int db = 0; db < 8; ++db)
 #pragma unroll
         for (int e = 0; e < 4; ++e) oacc[rb][db][e] = 0.f;
-      const bool ok = head_ok[rb];
-      const int64_t row =
-          ok ? ((int64_t)b * a.q_sb + (int64_t)(g * a.Gs + a.hoff + 8 * rb + grp) * a.q_sh) / 2 : 0;
-#pragma unroll
-      for (int kb = 0; kb < 8; ++kb) {
-        qa[rb][kb][0] = ok ? __ldg(q32 + row + kb * 8 + tig) : 0u;
-        qa[rb][kb][1] = ok ? __ldg(q32 + row + kb * 8 + 4 + tig) : 0u;
-      }
     }
+    if constexpr (!CL) load_q(b, g);
   };
 
   // write the current (b, g): the output itself when this segment holds all
   // of its batches, else a partial for the combine kernel
+  float* const staged = reinterpret_cast<float*>(asmem + (slot0 - smem_addr(asmem)));   // CL: in the warp's slot, free by then
   auto flush = [&]() {
-    const int nb_ = s_nbat[cu];
-    const int firstb = s_bstart[cu] + (a.kvh ? 0 : cg * nb_);   // first batch of (cb, cg) in the list
-    const bool whole = firstb / per == (firstb + nb_ - 1) / per;   // one segment holds it all
+    const int nb_ = nbat_of(cu);
+    const int firstb = CL ? 0 : s_bstart[cu] + (a.kvh ? 0 : cg * nb_);   // first batch of (cb, cg) in the list
+    const bool whole = !CL && firstb / per == (firstb + nb_ - 1) / per;   // one segment holds it all
     const int seg = gw - firstb / per;
 #pragma unroll
     for (int rb = 0; rb < kRB; ++rb) {
@@ -265,7 +337,7 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
         const int hl = 8 * rb + (c ? hB : hA);
         if (hl >= Gn) continue;
         const float m = c ? mB : mA, l = c ? lB : lA;
-        const int h = cg * a.Gs + a.hoff + hl;
+        const int h = cg * a.Gs + hoff + hl;
         if (whole) {
           float* op = a.out + ((int64_t)cb * a.H + h) * kHeadDim + grp;
           const float inv = l > 0.f ? 1.f / l : 0.f;
@@ -275,7 +347,7 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
             op[db * 16 + 8] = oacc[rb][db][2 + c] * inv;
           }
         } else {
-          float* pp = a.part + (((int64_t)cb * a.H + h) * a.splits + seg) * (2 + kHeadDim);
+          float* pp = CL ? staged + hl * kPS : a.part + (((int64_t)cb * a.H + h) * a.splits + seg) * kPS;
           if (grp == 0) {
             pp[0] = m;
             pp[1] = l;
@@ -418,7 +490,58 @@ __global__ void __launch_bounds__(kAThreads, 1) hill_sparse_attn_kernel(const __
     vm_cur = vm_next;
     advance(pc);
   }
-  flush();
+  if constexpr (!CL) {
+    flush();
+    return;
+  }
+  // CL: merge the warps' partials head by head; C > 1: push the CTA's to CTA
+  // h % C, which merges the CTAs'
+  if (t0 < t1) flush();
+  if (lane == 0) s_has[warp] = t0 < t1;
+  __syncthreads();
+  struct Acc {
+    float m = -INFINITY, l = 0.f, o[4] = {0.f, 0.f, 0.f, 0.f};   // dims lane + 32 i
+  };
+  auto fold = [&](Acc& x, const float* p) {
+    const float m = p[0], l = p[1];
+    if (m == -INFINITY) return;   // no token
+    const float mn = fmaxf(x.m, m), c0 = ex2(x.m - mn), c1 = ex2(m - mn);
+    x.l = x.l * c0 + l * c1;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x.o[i] = x.o[i] * c0 + p[2 + lane + 32 * i] * c1;
+    x.m = mn;
+  };
+  auto write_out = [&](const Acc& x, int hl) {
+    float* op = a.out + ((int64_t)tb * a.H + tg * a.Gs + hoff + hl) * kHeadDim + lane;
+    const float inv = x.l > 0.f ? 1.f / x.l : 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) op[32 * i] = x.o[i] * inv;
+  };
+  const float* const slots_f = staged - warp * (AttnCfg::kSlotBytes / 4);
+  if (C > 1) cg::this_cluster().barrier_wait();
+  for (int hl = warp; hl < Gn; hl += NW) {
+    Acc x;
+    for (int w = 0; w < NW; ++w)
+      if (s_has[w]) fold(x, slots_f + w * (AttnCfg::kSlotBytes / 4) + hl * kPS);
+    if (C == 1) {
+      write_out(x, hl);
+      continue;
+    }
+    float* d = cg::this_cluster().map_shared_rank(s_recv, hl % C) + ((hl / C) * C + rank) * kPS;
+    if (lane == 0) {
+      d[0] = x.m;
+      d[1] = x.l;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[2 + lane + 32 * i] = x.o[i];
+  }
+  if (C == 1) return;
+  cg::this_cluster().sync();
+  for (int i = warp; i * C + rank < Gn; i += NW) {
+    Acc x;
+    for (int c = 0; c < C; ++c) fold(x, s_recv + (i * C + c) * kPS);
+    write_out(x, i * C + rank);
+  }
 }
 
 // Merge the partials of one (b, h) whose batches were split over several
@@ -473,7 +596,6 @@ __global__ void __launch_bounds__(kCombThreads) hill_attn_combine_kernel(AttnArg
   const int per = (total + total_warps - 1) / total_warps;
   const int w0 = first / per, w1 = (first + nb - 1) / per;
   if (w0 == w1) return;   // one warp held every batch and wrote the output
-  constexpr int kPS = 2 + kHeadDim;   // one partial: max, sum, o[kHeadDim]
   const float* pp = a.part + (int64_t)bh * a.splits * kPS;
   const int nseg = w1 - w0 + 1;
   float M = -INFINITY, L = 0.f, O = 0.f;
@@ -530,12 +652,104 @@ __global__ void __launch_bounds__(kCombThreads) hill_attn_combine_kernel(AttnArg
 template <int DT, int G>
 cudaError_t launch_attn_t(const AttnArgs& a, int grid, bool combine, cudaStream_t st) {
   static int cache[64] = {0};
-  auto kern = hill_sparse_attn_kernel<DT, G>;
-  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), AttnCfg::kSmem, cache);
+  auto kern = hill_sparse_attn_kernel<DT, G, false, kAW>;
+  cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), AttnCfg::smem(kAW), cache);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(kern, dim3(grid), dim3(kAThreads), AttnCfg::kSmem, st, 0, a);
+  e = launch_pdl(kern, dim3(grid), dim3(kAThreads), AttnCfg::smem(kAW), st, 0, a);
   if (e != cudaSuccess || !combine) return e;
   return launch_pdl(hill_attn_combine_kernel, dim3(a.B * a.H), dim3(kCombThreads), 0, st, 0, a, grid * kAW);
+}
+
+// Clusters of C CTAs of the cluster form that the current device holds at once.
+template <int DT, int G, int NW>
+cudaError_t attn_clusters_fit(int C, int* n) {
+  static int cache[64] = {0};
+  static int fit[64][kMaxAttnCluster + 1];   // (+ 1; 0: not asked yet)
+  static std::mutex mu;
+  auto kern = hill_sparse_attn_kernel<DT, G, true, NW>;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  e = ensure_smem_attr(reinterpret_cast<const void*>(kern), AttnCfg::smem(NW), cache);   // (checks dev)
+  if (e != cudaSuccess) return e;
+  int& f = fit[dev][C];
+  if (f == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(C);
+    cfg.blockDim = dim3(NW * 32);
+    cfg.dynamicSmemBytes = AttnCfg::smem(NW);
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    e = cudaOccupancyMaxActiveClusters(&f, kern, &cfg);
+    if (e != cudaSuccess) return e;
+    ++f;
+  }
+  *n = f - 1;
+  return cudaSuccess;
+}
+
+// The largest cluster of CTAs of NW warps that all triples can have at once
+// (0: none), and the batches that a warp then takes at most.
+template <int DT, int G, int NW>
+cudaError_t attn_cluster_size(int64_t triples, int nb, int sms, int* C, int* rounds) {
+  *C = 0;
+  int c = (int)std::min<int64_t>({kMaxAttnCluster, (int64_t)sms * (kAW / NW) / triples, (nb + NW - 1) / NW});
+  for (; c >= 1; --c) {
+    int n = 0;
+    const cudaError_t e = attn_clusters_fit<DT, G, NW>(c, &n);
+    if (e != cudaSuccess) return e;
+    if (triples > n) continue;
+    *C = c;
+    *rounds = (nb + c * NW - 1) / (c * NW);
+    break;
+  }
+  return cudaSuccess;
+}
+
+// The cluster form, if it is the better one for this call (*done).
+template <int DT, int G>
+cudaError_t launch_attn_cl(const AttnArgs& a, int sms, cudaStream_t st, bool* done) {
+  *done = false;
+  const int64_t triples = (int64_t)a.B * a.Hkv * ((a.Gs + 15) / 16);
+  const int nb = (a.max_k + kBatch - 1) / kBatch;   // batches of a triple, at most
+  if (triples == 0 || nb == 0 || triples > 2 * sms) return cudaSuccess;
+  int c8 = 0, r8 = 0, c4 = 0, r4 = 0;
+  cudaError_t e = triples <= sms ? attn_cluster_size<DT, G, kAW>(triples, nb, sms, &c8, &r8) : cudaSuccess;
+  if (e == cudaSuccess) e = attn_cluster_size<DT, G, kAW / 2>(triples, nb, sms, &c4, &r4);
+  if (e != cudaSuccess) return e;
+  const bool half = c8 == 0 || (c4 > 0 && r4 < r8);
+  const int C = half ? c4 : c8, rounds = half ? r4 : r8;
+  const int64_t even = (triples * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
+  // A round (one more batch per warp) costs about 1.6 us where latency bounds
+  // it, the launches saved about 3.5 us and 8 more for every further pass over
+  // the heads; beyond some 10 rounds HBM bounds both forms until the uneven
+  // split shows.  Measured, even split / clusters (us, rounds in brackets):
+  // 32 heads, 8 x 4K k 20 % 25.0 / 20.0 (6 / 7), 4 x 16-32K k 10 % 34.7 / 32.2
+  // (11 / 13), 1 x 64K k 50 % 86.0 / 82.5 (27 / 33); 8 x 16-32K k 50 % 249 /
+  // 260 (108 / 129); 7 heads per KV head, 4 KV heads, 64K, k 10 % 12.4 / 10.3
+  // (1 / 4), k 20 % 14.2 / 14.9 (2 / 7); 32 heads on one KV head, k 20 % of
+  // 64K 24.7 / 18.7 (1 / 7), k 30 % of 128K 32.4 / 41.5 (3 / 20).
+  const int64_t passes = (a.Gs + 15) / 16;
+  if (C == 0 || even > 32 || rounds > even + even / 4 + 3 * passes) return cudaSuccess;
+  *done = true;
+  const dim3 grid((unsigned)(triples * C));
+  return half ? launch_pdl(hill_sparse_attn_kernel<DT, G, true, kAW / 2>, grid, dim3(kAThreads / 2), AttnCfg::smem(kAW / 2),
+                           st, C, a)
+              : launch_pdl(hill_sparse_attn_kernel<DT, G, true, kAW>, grid, dim3(kAThreads), AttnCfg::smem(kAW), st, C, a);
+}
+
+template <int DT>
+cudaError_t launch_attn_cl_d(const AttnArgs& a, int sms, cudaStream_t st, bool* done) {
+  if (a.Gs <= 1) return launch_attn_cl<DT, 1>(a, sms, st, done);
+  if (a.Gs <= 2) return launch_attn_cl<DT, 2>(a, sms, st, done);
+  if (a.Gs <= 4) return launch_attn_cl<DT, 4>(a, sms, st, done);
+  if (a.Gs <= 8) return launch_attn_cl<DT, 8>(a, sms, st, done);
+  return launch_attn_cl<DT, 16>(a, sms, st, done);
 }
 
 template <int DT>
@@ -558,6 +772,10 @@ int attn_max_batch() { return kMaxBatchAttn; }
 // Partial slots per (b, h): a (b, g) of nb batches meets at most
 // ceil(nb / per) + 1 warp segments, and per >= 1.
 int attn_max_segments(int max_k) { return (max_k + kBatch - 1) / kBatch + 1; }
+
+cudaError_t launch_sparse_attn_clusters(const AttnArgs& a, int dtype, int sms, cudaStream_t st, bool* done) {
+  return dtype == 0 ? launch_attn_cl_d<0>(a, sms, st, done) : launch_attn_cl_d<1>(a, sms, st, done);
+}
 
 cudaError_t launch_sparse_attn(const AttnArgs& a, int dtype, int G, int grid, bool combine, cudaStream_t st) {
   return dtype == 0 ? launch_attn_d<0>(a, G, grid, combine, st) : launch_attn_d<1>(a, G, grid, combine, st);

@@ -223,6 +223,9 @@ cudaError_t launch_select(const SelectArgs& a, int sms, cudaStream_t st);
 int attn_batch_tokens();
 int attn_max_batch();
 int attn_max_segments(int max_k);
+// The whole attention in one launch, a cluster of CTAs per (b, g, pass of 16
+// heads), where that is the better form (*done is set; a.hoff, a.Gn unused).
+cudaError_t launch_sparse_attn_clusters(const AttnArgs& a, int dtype, int sms, cudaStream_t st, bool* done);
 // The attention kernel for one pass of G heads per KV head, and (combine)
 // the merge of split partials over all heads.
 cudaError_t launch_sparse_attn(const AttnArgs& a, int dtype, int G, int grid, bool combine, cudaStream_t st);
