@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <atomic>
 #include <mutex>
+#include <random>
 
 #include "../../include/hill.h"
 #include "hill_internal.h"
@@ -33,6 +34,21 @@ std::atomic<uint64_t> g_launches{0};
 cudaError_t counted(cudaError_t e, int kernels) {
   if (e == cudaSuccess) g_launches.fetch_add((uint64_t)kernels, std::memory_order_relaxed);
   return e;
+}
+
+// The tag of a scoring launch whose tail is claimed: 63 random bits, odd (a
+// counter of the process from a random start, mixed; splitmix64, Steele et al.
+// 2014).
+unsigned long long next_claim_tag() {
+  static const uint64_t start = [] {
+    std::random_device rd;
+    return ((uint64_t)rd() << 32) ^ rd();
+  }();
+  static std::atomic<uint64_t> n{0};
+  uint64_t z = start + (n.fetch_add(1, std::memory_order_relaxed) + 1) * 0x9e3779b97f4a7c15ull;
+  z = (z ^ (z >> 30)) * 0xbf58476d1ce4e5b9ull;
+  z = (z ^ (z >> 27)) * 0x94d049bb133111ebull;
+  return (z ^ (z >> 31)) | 1ull;
 }
 
 // Per-device constants: SM count and the device address of the error word.
@@ -193,6 +209,9 @@ hill_status check_desc(const hill_desc* d) {
 struct Layout {
   size_t scores, logits, partials, stats, hist0, attn_part, q8, sq, total;
   bool has_hist0;
+  size_t claim;      // claim counters of the scoring kernel
+  bool has_claim;
+  int64_t nslot;     // ATTN partial slots per (b, h)
   int score_grid, attn_grid, splits;
   int score_spc;   // ATTN partial slots per scoring CTA
 };
@@ -229,6 +248,13 @@ Layout layout_for(const hill_desc* d, int mode, int max_k, int sms, bool score_o
   L.score_spc = d->num_kv_heads > score_max_kv_heads()
                     ? 1
                     : score_deal_warps(d->num_kv_heads, d->num_q_heads / d->num_kv_heads);
+  // the tail of a long K stream is claimed tile by tile (run_score); the
+  // allocation-free entry point keeps the even split and its documented scratch
+  L.has_claim = mode == HILL_SCORE_ATTN && e4m3_query && L.score_spc == 1 && !split_grid;
+  // (every unit that meets a sequence holds one of its tiles)
+  const int64_t tiles = std::max(1, (d->capacity + score_tile_tokens() - 1) / score_tile_tokens());
+  const int64_t units = L.has_claim ? score_claim_slots(d->batch * tiles, L.score_grid) : L.score_grid;
+  L.nslot = (e4m3_query ? std::min(tiles, units) : units) * L.score_spc;
   L.attn_grid = sms;
   L.splits = score_only ? 0 : attn_max_segments(max_k < 0 ? 0 : max_k);
   size_t off = 0;
@@ -239,7 +265,7 @@ Layout layout_for(const hill_desc* d, int mode, int max_k, int sms, bool score_o
   L.logits = off;
   if (mode == HILL_SCORE_ATTN) off += align_up(B * H * (size_t)cap32_of(d) * sizeof(float));
   L.partials = off;
-  if (mode == HILL_SCORE_ATTN) off += align_up(B * (size_t)L.score_grid * L.score_spc * H * sizeof(float2));
+  if (mode == HILL_SCORE_ATTN) off += align_up(B * (size_t)L.nslot * H * sizeof(float2));
   // combined (max, 1/sum) per (b, h), when the normalisation runs in two kernels
   L.stats = off;
   if (mode == HILL_SCORE_ATTN) off += align_up(B * H * sizeof(float2));
@@ -248,6 +274,8 @@ Layout layout_for(const hill_desc* d, int mode, int max_k, int sms, bool score_o
   L.hist0 = off;
   L.has_hist0 = mode == HILL_SCORE_ATTN && max_k > 0 && !score_only;
   if (L.has_hist0) off += align_up(B * (size_t)select_hist_bins() * sizeof(uint32_t));
+  L.claim = off;
+  if (L.has_claim) off += align_up(score_warps() * sizeof(ClaimCounter));
   L.attn_part = off;
   off += align_up(B * H * (size_t)L.splits * (2 + kHeadDim) * sizeof(float));
   // E4M3 query codes [B][Hkv][16][128] and scales [B][H]
@@ -299,6 +327,9 @@ hill_status head_passes(const hill_desc* d, bool kv_split, F&& f, int per_pass =
 // stream only (the scoring kernel), or the ATTN normalisation only.
 constexpr int kScoreAll = 0, kScoreStream = 1, kScoreNormalise = 2;
 
+// Key bytes from which the scoring kernel's tail is claimed (run_score).
+constexpr int64_t kClaimBytes = (int64_t)512 << 20;
+
 hill_status run_score(const hill_desc* d, const void* q, const void* k, const int32_t* lens, int mode,
                       float* scores, float* accum, unsigned char* base, const Layout& L,
                       const DeviceInfo& di, cudaStream_t st, uint32_t* hist0 = nullptr, int recent = 0,
@@ -318,7 +349,7 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   a.k_sb = d->k_sb;
   a.k_sh = d->k_sh;
   a.k_sn = d->k_sn;
-  a.nslot = L.score_grid * L.score_spc;
+  a.nslot = (int)L.nslot;
   a.err = di.err;
   // kscale != NULL: k is the E4M3 shadow of the keys (asymmetric-precision scoring)
   const bool f8 = kscale != nullptr;
@@ -348,6 +379,7 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   // or above the pass's heads (8 for the dealing kernel)
   const bool deal = L.score_spc > 1;
   a.Gs = G;
+  ClaimCounter* claim = L.has_claim ? reinterpret_cast<ClaimCounter*>(base + L.claim) : nullptr;
   // E4M3 scoring on the tensor cores' native 8-bit path (score_tc.cu) for
   // per-sequence importance with 2 to 16 query heads per KV head (at most
   // score_tc_max_heads() in all, one pass over the KV heads) and at least
@@ -399,6 +431,21 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
     if (ts == HILL_OK) ts = from_cuda(counted(launch_score_tc(t, raw, L.score_grid, st), 1));
     if (ts != HILL_OK || raw || part == kScoreStream) return ts;
   }
+  // The tail of a long 16-bit ATTN stream is claimed (score.cu).  Measured,
+  // hill_score, even split / claims (us): 268 MB of keys 42.3 / 46.8, 403 MB
+  // 63.7 / 63.8, 503 MB (40 KV heads) 80.7 / 80.6, 537 MB 83.0 / 79.9.  With 16 KV
+  // heads or fewer a warp has one or two boxes of a tile, too little to hide
+  // a claim's round trip (537 MB: 16 heads 89.8 / 91.3, 8 heads 94.8 / 96.8).  Not
+  // in the split step, whose streams follow one another without a gap (four
+  // pipelined layers 219.7 / 222.0 us), nor from the E4M3 shadow, whose stages are
+  // bound by the warps' own work (111.2 / 117.2).
+  const int64_t stream = (int64_t)d->batch * d->capacity * d->num_kv_heads * 2 * kHeadDim;
+  const bool claims = claim && part == kScoreAll && !f8 && G <= 8 && d->num_kv_heads <= score_max_kv_heads() &&
+                      d->num_kv_heads > 2 * score_warps() && stream >= kClaimBytes;
+  if (claims) {
+    a.claim = claim;
+    a.claim_tag = next_claim_tag();
+  }
   hill_status s = part == kScoreNormalise || tc ? HILL_OK : head_passes(d, true, [&](int goff, int nkv, int hoff,
                                                                                       int Gn, bool first) {
     a.goff = goff;
@@ -424,8 +471,11 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   f.B = d->batch;
   f.H = d->num_q_heads;
   f.cap = d->capacity;
-  f.nslot = L.score_grid * L.score_spc;
+  f.nslot = (int)L.nslot;
   f.spc = L.score_spc;
+  f.score_grid = L.score_grid;
+  f.claims = claims ? 1 : 0;
+  f.claim = claims ? claim : nullptr;
   f.scores = scores;
   f.accum = accum;
   f.hist0 = hist0;

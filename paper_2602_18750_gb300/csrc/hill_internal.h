@@ -11,6 +11,12 @@
 
 namespace hill {
 
+// A counter of claimed tiles (score.cu: open_claims).
+struct alignas(16) ClaimCounter {
+  unsigned long long tag;
+  unsigned count, pad;
+};
+
 struct ScoreArgs {
   CUtensorMap kmap;   // K cache: 4-D tiled map, 128-byte swizzle, box = 64 dims x kT tokens
                       // (E4M3 shadow: box = 128 codes x kT tokens)
@@ -27,7 +33,9 @@ struct ScoreArgs {
   float* logits;      // ATTN: [B][H][lstride] (lstride = cap rounded up to 32: a warp's 32 tokens of a head fill one 128-byte line)
   int64_t lstride;
   float2* partials;   // ATTN: [B][H][nslot] (max, sum 2^(z2 - max)), base-2 logits z2 = z * log2 e
-  int nslot;          // = grid size of the launch x score_deal_warps(nkv, G) (one slot per warp share)
+  int nslot;          // partial slots per (b, h): one per work unit (and warp share) that meets b
+  ClaimCounter* claim;   // ATTN: [score_warps()] counters of claims, or NULL: even split
+  unsigned long long claim_tag;   // of this launch (odd)
   int kvh;            // RAW with per-KV-head selection: scores/accum [B][Hkv][cap], summed over each group only
   // Query heads per KV head in the data (Gs), the first one this launch
   // handles (hoff) and how many (Gn, at most the kernel's template group G,
@@ -48,7 +56,10 @@ struct FinalizeArgs {
   const float2* partials;
   const int32_t* lens;
   int B, H, cap, nslot;
-  int spc;            // partial slots per scoring CTA (nslot = CTAs x spc)
+  int spc;            // partial slots per scoring unit
+  int score_grid;     // CTAs of the scoring launch
+  int claims;         // 1: its tail was claimed tile by tile (Units)
+  ClaimCounter* claim;   // the counters, closed here
   float* scores;      // may be NULL when accum is given
   float* accum;       // may be NULL
   uint32_t* hist0;    // optional [B][2048]: counts of the leading 11-bit digit of the selection key
@@ -182,6 +193,8 @@ cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
 
 // score.cu
 size_t score_smem_bytes(int G, bool f8);
+// Partial slots per (b, h) that a scoring launch with claims needs at most.
+int64_t score_claim_slots(int64_t n_items, int grid);
 int score_tile_tokens();
 int score_warps();
 int score_max_batch();

@@ -49,6 +49,9 @@ constexpr int kMaxNg = 4;                   // KV heads per warp per item (Hkv <
 constexpr int kBoxBytes = kT * 128;         // one 64-dim half of a tile: 32 swizzled 128-byte rows
 constexpr int kKBytes = 2 * kBoxBytes;
 
+constexpr int kShare16 = 13;   // sixteenths of the tiles dealt out in even shares when the rest is claimed
+constexpr int kFifo = 8;   // claimed tiles a warp can have in flight: at most kSW + 1
+
 template <int G, bool F8>
 struct ScoreCfg {
   // one K tile (a multiple of 1024): 8 KB of 16-bit keys, or 4 KB of E4M3 codes
@@ -62,7 +65,8 @@ struct ScoreCfg {
   static constexpr int kOffRed = kOffTab + 2 * kTableInts * 4;
   static constexpr int kOffFlag = kOffRed + 2 * kNW * kT * 4;
   static constexpr int kOffIssued = kOffFlag + kNW * 4;       // warps that issued their last stage
-  static constexpr int kBytes = kOffIssued + 16 + 1024;   // + alignment slack
+  static constexpr int kOffFifo = kOffIssued + 16;            // [kNW][kFifo] claimed tiles in flight
+  static constexpr int kBytes = kOffFifo + kNW * kFifo * 4 + 1024;   // + alignment slack
 };
 
 constexpr int kL2Ahead = 4;   // stages per warp brought into L2 before the dependency wait
@@ -81,6 +85,60 @@ __device__ __forceinline__ int find_seq(const int* tstart, int B, int item) {
   return lo;
 }
 
+// The tiles (items) of all sequences as work units.  Even split: CTA x takes
+// unit x, the items [x * per, (x + 1) * per).  With claims: unit x < grid is
+// the first share of CTA x, and every item from dyn0 on is a unit of its own,
+// claimed (per warp index, for that warp's heads) as warps become free.  A
+// sequence's partial slots are its units in order, so what a slot holds does
+// not depend on who claimed it.
+//
+// Why: SMs differ.  Those of a GPC with more SMs get less bandwidth each: per
+// CTA an even share of 4 x 16-32K tokens (32 heads) took 112 us in the median,
+// 120-127 on 40 of 152 SMs, and those alone do not fill HBM.  With 13/16 dealt
+// out and the rest claimed tile by tile: the whole step on 4 x 16-32K tokens
+// 178.8 -> 167.9 us, on 8 x 64K 887.9 -> 860.0 (11/16 and 12/16 the same within
+// 1 %, 14/16 2 % slower).  Opening the counters and a flush of the statistics
+// per claim cost 3-5 us, so short streams keep the even split (run_score).
+struct Units {
+  int per, dyn0, grid;   // items of a share; the first item claimed (INT_MAX: none)
+  __device__ __forceinline__ Units(int n_items, int grid_, bool claims) {
+    grid = grid_;
+    per = claims ? n_items / 16 * kShare16 / grid : (n_items + grid - 1) / grid;
+    dyn0 = claims ? grid * per : 0x7fffffff;
+  }
+  __device__ __forceinline__ int of(int item) const { return item < dyn0 ? item / per : grid + (item - dyn0); }
+};
+
+// The claim counters lie in the caller's workspace, whose contents are
+// arbitrary before a call, and no kernel of the call runs before this one.  So
+// the first warp that needs a counter opens it: a counter counts only under
+// the tag of its launch (odd, 64 random bits drawn by the host), which is put
+// in place in two steps (tag - 1 while the count is being zeroed).  The
+// normalisation, which runs when every claim is over, takes the tags away
+// again, so that a graph's next replay finds them closed.  A warp waits here
+// only for another one that is between two stores; the wait is bounded.
+__device__ __noinline__ void open_claims(ClaimCounter* c, unsigned long long tag, unsigned* err) {
+  volatile unsigned long long* t = &c->tag;
+  unsigned long long cur = *t;
+  if (cur != tag && cur != tag - 1) {
+    const unsigned long long seen = atomicCAS(&c->tag, cur, tag - 1);
+    if (seen == cur) {
+      *const_cast<volatile unsigned*>(&c->count) = 0u;
+      __threadfence();
+      *t = tag;
+      return;
+    }
+  }
+  const unsigned long long t0 = global_ns();
+  while (*t != tag) {
+    if (global_ns() - t0 > kWaitLimitNs) {
+      raise_error(err, kErrTimeout);
+      break;
+    }
+  }
+  __threadfence();
+}
+
 __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
@@ -92,7 +150,7 @@ struct Cursor {
   int item, r, b;
 };
 
-template <int DT, int G, bool RAW, bool F8, bool DEAL>
+template <int DT, int G, bool RAW, bool F8, bool DEAL, bool CLAIM>
 __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_constant__ ScoreArgs a) {
   using Cfg = ScoreCfg<G, F8>;
   constexpr int kSlotBytes = Cfg::kSlotBytes;
@@ -152,8 +210,10 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
   }
   __syncthreads();
   const int n_items = tstart[B];
-  const int per = (n_items + gridDim.x - 1) / gridDim.x;     // items per CTA
-  const int it_lo = min(n_items, (int)blockIdx.x * per), it_hi = min(n_items, it_lo + per);
+  static_assert(!CLAIM || (!RAW && !DEAL && !F8), "tiles are claimed on the 16-bit ATTN stream");
+  const Units units(n_items, gridDim.x, CLAIM);
+  const int per = units.per;
+  const int it_lo = min(n_items, (int)blockIdx.x * per), it_hi = min(n_items, it_lo + per);   // this CTA's share
   // The warps' shares.  Without DEAL (W = 1) the KV heads are dealt to the
   // warps -- warp w takes g0 + r * kNW, r < ng (0 .. kMaxNg) -- and every warp
   // visits every item of the CTA.  With DEAL (launches of at most kNW / 2 KV
@@ -191,6 +251,45 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
       while (c.b < B - 1 && tstart[c.b + 1] <= c.item) ++c.b;
     }
   };
+  // Past its share a warp CLAIM single tiles for its heads from the counter
+  // of its warp index (lane 0; the claim made one tile ahead, so that its
+  // round trip is over when it is needed), and notes them for the consumer.
+  int* fifo = reinterpret_cast<int*>(base + Cfg::kOffFifo) + warp * kFifo;
+  unsigned claimed = 0, taken = 0;   // claims of the cursor, and of these taken by the consumer
+  unsigned ahead = 0;                // lane 0: the claim made ahead
+  bool is_ahead = false, opened = false;
+  auto claim_ahead = [&]() {
+    if (!opened) {
+      if (lane == 0) open_claims(a.claim + warp, a.claim_tag, a.err);
+      opened = true;
+    }
+    if (lane == 0) ahead = atomicAdd(&a.claim[warp].count, 1u);
+    is_ahead = true;
+  };
+  auto claim = [&](Cursor& c) {      // c.item = the next claimed tile, or n_items
+    if (!is_ahead) claim_ahead();
+    const unsigned u = __shfl_sync(0xffffffffu, ahead, 0);
+    c.r = 0;
+    if (u >= (unsigned)(n_items - units.dyn0)) {
+      c.item = n_items;
+      return;
+    }
+    c.item = units.dyn0 + (int)u;
+    while (c.b < B - 1 && tstart[c.b + 1] <= c.item) ++c.b;
+    if (lane == 0) fifo[claimed % kFifo] = c.item;
+    ++claimed;
+    claim_ahead();
+  };
+  // the cursor's next stage: of its item, its share or a claimed tile
+  const int it_end = CLAIM ? n_items : it_hi;   // where the cursor ends
+  auto next_stage = [&](Cursor& c) {
+    if (!CLAIM || c.r + 1 < ng || c.item + 1 < it_hi) {
+      advance(c);
+      if (CLAIM && c.item + 1 == it_hi && c.r == 0) claim_ahead();
+    } else {
+      claim(c);
+    }
+  };
   // lane 0: load the K tile of position c into slot s
   auto issue = [&](const Cursor& c, uint32_t s) {
     const int j0 = (c.item - tstart[c.b]) * kT;
@@ -222,7 +321,7 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
   // step, measured slower so and keeps the release at exit
   bool marked = F8;
   auto mark_if_done = [&]() {
-    if (!marked && (ng == 0 || pc.item >= it_hi)) {
+    if (!marked && (ng == 0 || pc.item >= it_end)) {
       marked = true;
       if (lane == 0 && atomicAdd(reinterpret_cast<int*>(base + Cfg::kOffIssued), 1) == kNW - 1)
         pdl_launch_dependents();
@@ -268,8 +367,17 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
     const int64_t w1 = min(w0 + hper, a.hist0_words);
     for (int64_t w = w0 + threadIdx.x; w < w1; w += kThreads) a.hist0[w] = 0u;
   }
-  if (it_lo >= it_hi) return;
+  if (CLAIM ? n_items == 0 : it_lo >= it_hi) return;
   if constexpr (F8) prologue();
+  if (CLAIM && ng > 0 && pc.item >= it_hi) {   // a share shorter than the ring: go on with CLAIM
+    claim(pc);
+    while (issued < (uint32_t)kSW && pc.item < n_items) {
+      if (lane == 0) issue(pc, is_slot);
+      ++issued;
+      is_slot = is_slot + 1 == (uint32_t)kSW ? 0u : is_slot + 1;
+      next_stage(pc);
+    }
+  }
   mark_if_done();
 
   // fragment coordinates (mma.sync m16n8k16): C row = token lane/4 (+8),
@@ -281,7 +389,7 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
   uint32_t used = 0, cs = 0, cph = 0;      // stages consumed; slot and phase of the next one
   int item_no = 0;
   bool ok = true;
-  int cur_b = -1, cur_slot = 0;
+  int cur_b = -1, cur_unit = -1, cur_slot = 0;
 
   // q of this warp's heads for the current sequence, as mma B fragments:
   // column grp is query head g*Gs + hoff + grp (zero for grp >= Gn), k = 16*kb + 2*tig (+8)
@@ -394,23 +502,32 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
     }
   };
 
-  for (int item = it0, b = b_first; item < it_hi; item += W, ++item_no) {
+  for (int own = it0, b = b_first;; own += W, ++item_no) {
+    int item = own;
+    if (own >= it_hi) {   // the share is done: the claimed tiles, in order
+      if constexpr (!CLAIM) break;
+      if (taken == claimed) break;
+      __syncwarp();
+      item = fifo[taken++ % kFifo];
+    }
     while (b < B - 1 && tstart[b + 1] <= item) ++b;
     const int tile = item - tstart[b];
     const int j0 = tile * kT;
     const int nv = min(kT, slen[b] - j0);
     float rs[4] = {0.f, 0.f, 0.f, 0.f};   // RAW: token sums of rows grp, grp+8, 16+grp, 24+grp
 
-    if (b != cur_b) {
+    const int unit = own < it_hi ? (int)blockIdx.x : units.of(item);
+    if (b != cur_b || (CLAIM && unit != cur_unit)) {
       if (!RAW && cur_b >= 0) flush();
       neutral_until(b);
       b_next = b + 1;
-      load_q(b);
+      if (b != cur_b) load_q(b);
       if (!RAW) reset_stat();
       cur_b = b;
-      // this warp's partial slot in b: the CTA's rank among the CTAs whose
-      // ranges meet b, times W, plus the warp's item share
-      cur_slot = ((int)blockIdx.x - tstart[b] / per) * W + sub;
+      cur_unit = unit;
+      // this warp's partial slot in b: the unit's rank among the units that
+      // meet b, times W, plus the warp's item share
+      cur_slot = (unit - units.of(tstart[b])) * W + sub;
     }
 
     constexpr int kStagesPerItem = DEAL ? 1 : kMaxNg;   // (at most; ng of them)
@@ -454,13 +571,13 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
       const uint32_t freed = cs;
       cs = cs + 1 == (uint32_t)kSW ? 0u : cs + 1;
       __syncwarp();
-      if (pc.item < it_hi) {   // the slot just read takes the stage kSW ahead
+      if (pc.item < it_end) {   // the slot just read takes the stage kSW ahead
         if (lane == 0) {
           fence_proxy_async_smem();
           issue(pc, freed);
         }
         ++issued;
-        advance(pc);
+        next_stage(pc);
         mark_if_done();
       }
 
@@ -689,12 +806,12 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
   }
   __syncthreads();
   const int first_item = s_first;
-  const int grid = a.nslot / a.spc;   // CTAs of the scoring launch
-  const int per = (s_total + grid - 1) / grid;
+  const Units units(s_total, a.score_grid, a.claims != 0);
   const int items = (len + kT - 1) / kT;
-  const int ns = ((first_item + items - 1) / per - first_item / per + 1) * a.spc;
+  const int ns = (units.of(first_item + items - 1) - units.of(first_item) + 1) * a.spc;
   pdl_wait();
   pdl_launch_dependents();
+  if (a.claim && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kNW) a.claim[threadIdx.x].tag = 0ull;
   // This token's logits of heads [h0, h0 + kFinZ), 8 at a time (those past H
   // repeat the last head, with weight 0).  Threads past the length read the
   // last token's and write nothing.
@@ -799,19 +916,22 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
   }
 }
 
-// Combine the per-CTA (max, sum) partials of one (b, h) into its softmax
-// statistics (max, 1 / sum) in the base-2 scale: one warp per pair, each lane
-// taking every 32nd partial with a running maximum, the lanes then merged by
-// shuffles.  Used ahead of hill_attn_finalize_kernel<true, *> when the
-// normalisation has many CTAs per sequence.
+// Combine the per-unit (max, sum) partials of one (b, h) into its softmax
+// statistics (max, 1 / sum) in the base-2 scale: W warps per pair, each lane
+// taking every 32 W-th partial with a running maximum, the lanes then merged
+// by shuffles and the warps in shared memory.  Used ahead of
+// hill_attn_finalize_kernel<true, *> when the normalisation has many CTAs per
+// sequence; W > 1 when tiles were claimed, which leaves a partial per tile.
 constexpr int kStatsWarps = 8;
 constexpr int kStatsPer = 8;   // partials per lane whose loads are in flight together
 
+template <int W>
 __global__ void __launch_bounds__(kStatsWarps * 32) hill_attn_stats_kernel(FinalizeArgs a) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int pair = blockIdx.x * kStatsWarps + warp;
-  if (pair >= a.B * a.H) return;
-  const int b = pair / a.H;
+  __shared__ float2 s_part[kStatsWarps];
+  const int pair = (blockIdx.x * kStatsWarps + warp) / W, sub = warp % W;
+  const bool live = pair < a.B * a.H;
+  const int b = live ? pair / a.H : 0;
   // the slots 0 .. ns-1 of b (lengths are inputs of the call: read before the wait)
   int f = 0, t = 0;
   for (int bb = lane; bb < a.B; bb += 32) {
@@ -829,18 +949,17 @@ __global__ void __launch_bounds__(kStatsWarps * 32) hill_attn_stats_kernel(Final
   int len = a.lens[b];
   len = len < 0 ? 0 : (len > a.cap ? a.cap : len);
   const int items = (len + kT - 1) / kT;
-  const int grid = a.nslot / a.spc;   // CTAs of the scoring launch
-  const int per = (t + grid - 1) / grid;
-  const int ns = items == 0 ? 0 : ((f + items - 1) / per - f / per + 1) * a.spc;
+  const Units units(t, a.score_grid, a.claims != 0);
+  const int ns = items == 0 || !live ? 0 : (units.of(f + items - 1) - units.of(f) + 1) * a.spc;
   pdl_wait();
   pdl_launch_dependents();
   const float2* pb = a.partials + (int64_t)pair * a.nslot;
   float m = -INFINITY, l = 0.f;
-  for (int s0 = lane; s0 < ns; s0 += 32 * kStatsPer) {
+  for (int s0 = sub * 32 + lane; s0 < ns; s0 += 32 * W * kStatsPer) {
     float2 p[kStatsPer];
 #pragma unroll
     for (int u = 0; u < kStatsPer; ++u) {
-      const int s = s0 + 32 * u;
+      const int s = s0 + 32 * W * u;
       p[u] = s < ns ? pb[s] : make_float2(-INFINITY, 0.f);
     }
 #pragma unroll
@@ -851,21 +970,29 @@ __global__ void __launch_bounds__(kStatsWarps * 32) hill_attn_stats_kernel(Final
       m = mn;
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float mo = __shfl_xor_sync(0xffffffffu, m, o);
-    const float lo = __shfl_xor_sync(0xffffffffu, l, o);
+  auto merge = [&](float mo, float lo) {
     const float mn = fmaxf(m, mo);
     l = (l > 0.f ? l * ex2(m - mn) : 0.f) + (lo > 0.f ? lo * ex2(mo - mn) : 0.f);
     m = mn;
+  };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float mo = __shfl_xor_sync(0xffffffffu, m, o), lo = __shfl_xor_sync(0xffffffffu, l, o);
+    merge(mo, lo);
   }
-  if (lane == 0) a.stats[pair] = make_float2(m, 1.f / l);
+  if constexpr (W > 1) {
+    if (lane == 0) s_part[warp] = make_float2(m, l);
+    __syncthreads();
+    if (sub == 0)
+      for (int w = 1; w < W; ++w) merge(s_part[warp + w].x, s_part[warp + w].y);
+  }
+  if (live && sub == 0 && lane == 0) a.stats[pair] = make_float2(m, 1.f / l);
 }
 
-template <int DT, int G, bool RAW, bool F8, bool DEAL>
+template <int DT, int G, bool RAW, bool F8, bool DEAL, bool CLAIM = false>
 cudaError_t launch_score_t(const ScoreArgs& a, int grid, cudaStream_t st) {
   const size_t smem = (size_t)ScoreCfg<G, F8>::kBytes;
-  auto kern = hill_score_kernel<DT, G, RAW, F8, DEAL>;
+  auto kern = hill_score_kernel<DT, G, RAW, F8, DEAL, CLAIM>;
   static int cache[64] = {0};
   cudaError_t e = ensure_smem_attr(reinterpret_cast<const void*>(kern), (int)smem, cache);
   if (e != cudaSuccess) return e;
@@ -875,6 +1002,17 @@ cudaError_t launch_score_t(const ScoreArgs& a, int grid, cudaStream_t st) {
 template <int DT, bool RAW, bool F8>
 cudaError_t launch_score_g(const ScoreArgs& a, int G, bool deal, int grid, cudaStream_t st) {
   if (deal) return G == 8 ? launch_score_t<DT, 8, RAW, F8, true>(a, grid, st) : cudaErrorInvalidValue;
+  if constexpr (!RAW && !F8) {
+    if (a.claim) {
+      switch (G) {
+        case 1: return launch_score_t<DT, 1, RAW, F8, false, true>(a, grid, st);
+        case 2: return launch_score_t<DT, 2, RAW, F8, false, true>(a, grid, st);
+        case 4: return launch_score_t<DT, 4, RAW, F8, false, true>(a, grid, st);
+        case 8: return launch_score_t<DT, 8, RAW, F8, false, true>(a, grid, st);
+      }
+      return cudaErrorInvalidValue;
+    }
+  }
   switch (G) {
     case 1: return launch_score_t<DT, 1, RAW, F8, false>(a, grid, st);
     case 2: return launch_score_t<DT, 2, RAW, F8, false>(a, grid, st);
@@ -901,6 +1039,7 @@ size_t score_smem_bytes(int G, bool f8) {
   }
 }
 
+int64_t score_claim_slots(int64_t n_items, int grid) { return 2 * (int64_t)grid + n_items * 3 / 16 + 32; }
 int score_tile_tokens() { return kT; }
 int score_warps() { return kNW; }
 int score_max_batch() { return kMaxBatchSmem; }
@@ -941,9 +1080,10 @@ cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t s
   // SM the second launch costs more than it saves (about 2 us).
   if (two_kernel || (long long)a.B * ((a.cap + kFinThreads - 1) / kFinThreads) > sms) {
     *kernels = 2;
-    const int pairs = a.B * a.H;
-    cudaError_t e = launch_pdl(hill_attn_stats_kernel, dim3((pairs + kStatsWarps - 1) / kStatsWarps),
-                               dim3(kStatsWarps * 32), 0, st, 0, a);
+    const int W = a.claims ? 4 : 1;   // warps per (b, h)
+    const dim3 sgrid((a.B * a.H * W + kStatsWarps - 1) / kStatsWarps);
+    cudaError_t e = W > 1 ? launch_pdl(hill_attn_stats_kernel<4>, sgrid, dim3(kStatsWarps * 32), 0, st, 0, a)
+                          : launch_pdl(hill_attn_stats_kernel<1>, sgrid, dim3(kStatsWarps * 32), 0, st, 0, a);
     return e != cudaSuccess ? e : launch_finalize_t<true>(a, st);
   }
   *kernels = 1;

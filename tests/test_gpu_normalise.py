@@ -53,3 +53,38 @@ def test_scores_and_selection(case):
         # the selection is exact on the kernel's own sums
         order = torch.sort(accum[b, :m], descending=True, stable=True).indices[:kept[b]]
         assert torch.equal(idx[b, :kept[b]].long(), order.sort().values)
+
+
+@pytest.mark.parametrize("lens", [[7100] * 8, [7100, 0, 1, 31, 32, 33, 4000, 7099], [0, 0, 0, 0, 0, 0, 0, 200],
+                                  [5000, 0, 0, 0, 0, 0, 0, 0], [640, 641, 639, 7, 0, 0, 1500, 3]])
+@pytest.mark.parametrize("Hq,Hkv", [(32, 32), (64, 32), (48, 16)])
+def test_claimed_tail_of_a_large_cache(Hq, Hkv, lens):
+    """A cache large enough for the scoring kernel's tail to be claimed, full, ragged and nearly empty (shares shorter
+    than a warp's ring, no share at all): right against float64 and the same bits every time."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_18750_gb300 import build, hill as H
+    build.build()
+    B, cap, G = 8, 7168 * 32 // Hkv, Hq // Hkv
+    g = torch.Generator(device="cuda").manual_seed(sum(lens) + Hq)
+    K = torch.empty(B, Hkv, cap, 128, dtype=torch.bfloat16, device="cuda")
+    for b, m in enumerate(lens):
+        K[b, :, :m] = torch.randn(Hkv, m, 128, generator=g, device="cuda").bfloat16()
+        K[b, :, m:] = float("nan")
+    q = (2 * torch.randn(B, Hq, 128, generator=g, device="cuda")).bfloat16()
+    desc = H.make_desc(q, K)
+    lens_t = torch.tensor(lens, dtype=torch.int32, device="cuda")
+    ws = H.alloc_workspace(desc, 0, 0)
+    first = None
+    for fill in (0, 0xFF, 0x5A):
+        ws.fill_(fill)
+        scores = torch.zeros(B, cap, device="cuda")
+        H.hill_score(desc, q, K, lens_t, 0, scores, None, ws)
+        H.hill_sync_status()
+        assert first is None or torch.equal(scores, first)
+        first = scores
+    for b, m in enumerate(lens):
+        z = torch.stack([K[b, h // G, :m].double() @ q[b, h].double() for h in range(Hq)]) / np.sqrt(128)
+        ref = torch.softmax(z, -1).sum(0)
+        assert m == 0 or torch.all((scores[b, :m].double() - ref).abs() <= 2e-5 * ref)
+        assert not scores[b, m:].any()
