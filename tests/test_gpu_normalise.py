@@ -55,6 +55,32 @@ def test_scores_and_selection(case):
         assert torch.equal(idx[b, :kept[b]].long(), order.sort().values)
 
 
+@pytest.mark.parametrize("H_,Hkv", [(6, 3), (12, 3), (20, 20), (9, 3), (72, 9), (48, 2), (40, 8)])
+def test_group_sums(H_, Hkv):
+    """Per-KV-head importance for groups of 1, 2, 4, 8, 24 and odd sizes, head counts that are no multiple of 8."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_18750_gb300 import build, hill as H
+    build.build()
+    B, n, G, lens = 2, 700, H_ // Hkv, [700, 333]
+    g = torch.Generator(device="cuda").manual_seed(H_)
+    K = torch.randn(B, Hkv, n, 128, generator=g, device="cuda").half()
+    q = (2 * torch.randn(B, H_, 128, generator=g, device="cuda")).half()
+    desc = H.make_desc(q, K)
+    dev = lambda v: torch.tensor(v, dtype=torch.int32, device="cuda")  # noqa: E731
+    scores = torch.zeros(B, Hkv, n, device="cuda")
+    idx = torch.zeros(B, Hkv, 70, dtype=torch.int32, device="cuda")
+    count = torch.zeros(B, Hkv, dtype=torch.int32, device="cuda")
+    H.hill_evict_step_kvh(desc, q, K, None, dev(lens), dev([70, 33]), 70, 0, None, scores, idx, count, None,
+                          H.alloc_workspace(desc, 0, 70))
+    H.hill_sync_status()
+    for b, m in enumerate(lens):
+        z = torch.stack([K[b, h // G, :m].double() @ q[b, h].double() for h in range(H_)]) / np.sqrt(128)
+        ref = torch.softmax(z, -1).reshape(Hkv, G, m).sum(1)
+        assert torch.all((scores[b, :, :m].double() - ref).abs() <= 2e-5 * ref)
+        assert not scores[b, :, m:].any()
+
+
 @pytest.mark.parametrize("lens", [[7100] * 8, [7100, 0, 1, 31, 32, 33, 4000, 7099], [0, 0, 0, 0, 0, 0, 0, 200],
                                   [5000, 0, 0, 0, 0, 0, 0, 0], [640, 641, 639, 7, 0, 0, 1500, 3]])
 @pytest.mark.parametrize("Hq,Hkv", [(32, 32), (64, 32), (48, 16)])
