@@ -251,7 +251,7 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
       while (c.b < B - 1 && tstart[c.b + 1] <= c.item) ++c.b;
     }
   };
-  // Past its share a warp CLAIM single tiles for its heads from the counter
+  // Past its share a warp claims single tiles for its heads from the counter
   // of its warp index (lane 0; the claim made one tile ahead, so that its
   // round trip is over when it is needed), and notes them for the consumer.
   int* fifo = reinterpret_cast<int*>(base + Cfg::kOffFifo) + warp * kFifo;
@@ -369,7 +369,7 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
   }
   if (CLAIM ? n_items == 0 : it_lo >= it_hi) return;
   if constexpr (F8) prologue();
-  if (CLAIM && ng > 0 && pc.item >= it_hi) {   // a share shorter than the ring: go on with CLAIM
+  if (CLAIM && ng > 0 && pc.item >= it_hi) {   // a share shorter than the ring: go on with claims
     claim(pc);
     while (issued < (uint32_t)kSW && pc.item < n_items) {
       if (lane == 0) issue(pc, is_slot);
