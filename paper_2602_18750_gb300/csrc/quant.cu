@@ -17,7 +17,8 @@
 // rows, 640 MB moved): 91 us, 7.07 TB/s, where one row per warp and 8 bytes
 // per lane (one CTA per 8 rows) took 280 us.  Other splits: 2 rows per lane
 // 96-101 us, 1 row 119; 16 lanes per row 113-126; a persistent grid that
-// prefetches the next rows 111-139.
+// prefetches the next rows 111-139.  A few rows keep one row per warp
+// (launch_quantize_k).
 #include <type_traits>
 
 #include "hill_internal.h"
@@ -28,6 +29,7 @@ namespace {
 constexpr int kQWarps = 8;
 constexpr int kQU = 4;                // rows per quarter-warp
 constexpr int kQRows = 4 * kQU;       // rows per warp
+constexpr int kQFew = 6144;           // up to this many rows in all: one row per warp
 
 struct Dims16 {
   uint32_t v[8];   // 16 dims of a row
@@ -114,6 +116,40 @@ __global__ void __launch_bounds__(kQWarps * 32, 4) hill_quantize_k_kernel(const 
   }
 }
 
+// One row per warp, 8 bytes per lane, for calls of a few rows (the new tokens
+// of a step): bound by latency, they want a short chain in each warp.
+template <int DT>
+__global__ void __launch_bounds__(kQWarps * 32) hill_quantize_k_rows_kernel(const QuantArgs a) {
+  pdl_wait();
+  pdl_launch_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int b = blockIdx.z, g = blockIdx.y;
+  int j0 = a.row_begin[b], j1 = a.row_end[b];
+  j0 = j0 < 0 ? 0 : (j0 > a.cap ? a.cap : j0);
+  j1 = j1 < j0 ? j0 : (j1 > a.cap ? a.cap : j1);
+  const int j = j0 + blockIdx.x * kQWarps + warp;
+  if (j >= j1) return;
+  const auto* kr = static_cast<const uint16_t*>(a.k) + (int64_t)b * a.k_sb + (int64_t)g * a.k_sh + (int64_t)j * a.k_sn;
+  const uint2 raw = *reinterpret_cast<const uint2*>(kr + lane * 4);
+  const float2 x = unpack2<DT>(raw.x), y = unpack2<DT>(raw.y);
+  float amax = fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(y.x), fabsf(y.y)));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  const int64_t bg = (int64_t)b * a.Hkv + g;
+  const bool pos = amax > 0.f;
+  const float r = pos ? __fdiv_rn(448.f, amax) : 0.f;
+  const uint32_t code =
+      e4m3x2(__fmul_rn(x.x, r), __fmul_rn(x.y, r)) | (e4m3x2(__fmul_rn(y.x, r), __fmul_rn(y.y, r)) << 16);
+  reinterpret_cast<uint32_t*>(a.k8 + (bg * a.cap + j) * kHeadDim)[lane] = pos ? code : 0u;
+  if (lane == 0) a.kscale[bg * a.cap32 + j] = pos ? __fdiv_rn(amax, 448.f) : 0.f;
+}
+
+template <int DT>
+cudaError_t launch_quantize_rows(const QuantArgs& a, int max_rows, cudaStream_t st) {
+  return launch_pdl(hill_quantize_k_rows_kernel<DT>, dim3((max_rows + kQWarps - 1) / kQWarps, a.Hkv, a.B),
+                    dim3(kQWarps * 32), 0, st, 0, a);
+}
+
 template <int DT, bool A32>
 cudaError_t launch_quantize_t(const QuantArgs& a, cudaStream_t st) {
   const int64_t warps = (int64_t)a.B * a.Hkv * a.chunks;
@@ -125,6 +161,11 @@ cudaError_t launch_quantize_t(const QuantArgs& a, cudaStream_t st) {
 
 cudaError_t launch_quantize_k(const QuantArgs& a0, int dtype, int max_rows, cudaStream_t st) {
   QuantArgs a = a0;
+  // one row per warp / 16 rows per warp (us, in a graph): 8 (b, g) of 1 row 1.37 / 1.73, of 128 rows 1.52 / 2.13; 128 of
+  // 16 rows 1.59 / 2.16, of 32 1.95 / 2.16, of 64 2.36 / 2.22; 256 of 24 rows 2.25 / 2.21, of 64 3.28 / 2.31: the line
+  // is at about 40 rows per SM
+  if ((int64_t)a.B * a.Hkv * max_rows <= kQFew)
+    return dtype == 0 ? launch_quantize_rows<0>(a, max_rows, st) : launch_quantize_rows<1>(a, max_rows, st);
   a.chunks = (max_rows + kQRows - 1) / kQRows;
   // rows that all start on 32 bytes are read with 32-byte loads (91 us on the
   // case above); the interface asks for 16 only, and those take two 16-byte

@@ -70,12 +70,14 @@ def test_quantize_k_bit_exact(H, oracle_mod, dtype):
 
 @pytest.mark.parametrize("dtype", [torch.float16, torch.bfloat16])
 @pytest.mark.parametrize("pad", [0, 8, 16])
-@pytest.mark.parametrize("rows", [1, 3, 4, 5, 15, 16, 17, 33])
-def test_quantize_k_row_counts(H, oracle_mod, rows, pad, dtype):
+@pytest.mark.parametrize("rows", [1, 3, 4, 5, 15, 16, 17, 33, 682, 683])
+@pytest.mark.parametrize("bound", ["rows", "capacity"])
+def test_quantize_k_row_counts(H, oracle_mod, bound, rows, pad, dtype):
     """Row counts at the edges of a warp's 16 rows, rows that start on 32 bytes and rows that start on 16 only,
     subnormal values: exactly the requested rows are written, bit for bit, also where the sequences ask for different
-    counts under one max_rows."""
-    B, Hkv, cap = 3, 3, 60
+    counts under one max_rows. With the capacity as max_rows, 9 * 690 rows are past the 6144 up to which a warp takes
+    one row; 683 rows are the first count past it."""
+    B, Hkv, cap = 3, 3, 690
     g = torch.Generator().manual_seed(rows)
     K = torch.randn(B, Hkv, cap, 128, generator=g)
     # rows of subnormals in fp16; in bf16 as small as a row may be: 448 / amax has to be finite in float32, so
@@ -91,7 +93,7 @@ def test_quantize_k_row_counts(H, oracle_mod, rows, pad, dtype):
     ks.fill_(-1.0)
     begin = [5, cap - rows, 0]
     end = [5 + rows, cap, rows // 2]
-    H.hill_quantize_k(desc, Kd, _i32(begin), _i32(end), rows, k8, ks)
+    H.hill_quantize_k(desc, Kd, _i32(begin), _i32(end), rows if bound == "rows" else cap, k8, ks)
     H.hill_sync_status()
     codes, scale = oracle_mod.quantize_rows(K)
     got_c, got_s = k8.cpu().numpy(), ks.cpu().numpy()
