@@ -787,7 +787,19 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
   len = len < 0 ? 0 : (len > a.cap ? a.cap : len);
   // this CTA's tokens: a.tpt blocks of kFinThreads from jb
   const int jb = blockIdx.x * kFinThreads * a.tpt;
-  if (jb >= len) return;
+  // CTA (0, 0) closes the claim counters whatever its sequence's length, and
+  // always waits: so this grid never completes before the ones ahead of it,
+  // and a later call's claims never meet this call's closing
+  auto close_claims = [&]() {
+    if (a.claim && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kNW) a.claim[threadIdx.x].tag = 0ull;
+  };
+  if (jb >= len) {
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+      pdl_wait();
+      close_claims();
+    }
+    return;
+  }
   // the scoring CTAs that met b wrote slots 0 .. ns-1
   // (every thread counts the tiles of a share of the sequences)
   __shared__ int s_first, s_total;
@@ -815,7 +827,7 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
   const int ns = (units.of(first_item + items - 1) - units.of(first_item) + 1) * a.spc;
   pdl_wait();
   pdl_launch_dependents();
-  if (a.claim && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < kNW) a.claim[threadIdx.x].tag = 0ull;
+  close_claims();
   // This token's logits of heads [h0, h0 + kFinZ), 8 at a time (those past H
   // repeat the last head, with weight 0).  Threads past the length read the
   // last token's and write nothing.

@@ -114,3 +114,56 @@ def test_claimed_tail_of_a_large_cache(Hq, Hkv, lens):
         ref = torch.softmax(z, -1).sum(0)
         assert m == 0 or torch.all((scores[b, :m].double() - ref).abs() <= 2e-5 * ref)
         assert not scores[b, m:].any()
+
+
+@pytest.mark.parametrize("Hq,Hkv,cap", [(32, 32, 24000), (48, 24, 32000)])
+@pytest.mark.parametrize("fused", [False, True])
+def test_claims_in_a_replayed_graph(fused, Hq, Hkv, cap):
+    """A call whose tail is claimed, captured once and replayed over lengths and queries that change between the
+    replays, the first sequence, all of them or none empty: every replay gives the bits of an eager call on a workspace
+    of its own."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_18750_gb300 import build, hill as H
+    build.build()
+    B, max_k = 4, 64
+    g = torch.Generator(device="cuda").manual_seed(cap)
+    K = torch.randn(B, Hkv, cap, 128, generator=g, device="cuda").bfloat16()
+    q = torch.empty(B, Hq, 128, dtype=torch.bfloat16, device="cuda")
+    desc = H.make_desc(q, K)
+    lens = torch.full((B,), cap, dtype=torch.int32, device="cuda")
+    k = torch.full((B,), max_k, dtype=torch.int32, device="cuda")
+
+    def buffers():
+        ws = H.alloc_workspace(desc, 0, max_k)
+        ws.fill_(0x5A)
+        return {"ws": ws, "scores": torch.zeros(B, cap, device="cuda"), "accum": torch.zeros(B, cap, device="cuda"),
+                "idx": torch.zeros(B, max_k, dtype=torch.int32, device="cuda"),
+                "count": torch.zeros(B, dtype=torch.int32, device="cuda")}
+
+    def call(y):
+        if fused:
+            H.hill_evict_step(desc, q, K, None, lens, k, max_k, 0, y["accum"], y["scores"], y["idx"], y["count"], None,
+                              y["ws"])
+        else:
+            H.hill_score(desc, q, K, lens, 0, y["scores"], y["accum"], y["ws"])
+
+    call(buffers())   # (kernels loaded)
+    H.hill_sync_status()
+    y = buffers()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call(y)
+    empty, full = [0] * B, [cap] * B
+    first = [0] + [cap] * (B - 1)
+    for step, n in enumerate([full, first, full, first, first, empty, full, [cap, 0, cap - 33, cap], [0, 0, 0, cap], full]):
+        q.copy_(2 * torch.randn(q.shape, generator=g, device="cuda"))
+        lens.copy_(torch.tensor(n, dtype=torch.int32))
+        want = buffers()
+        for o in ("scores", "accum"):
+            want[o].copy_(y[o])
+        call(want)
+        graph.replay()
+        H.hill_sync_status()
+        for o in ("scores", "accum", "idx", "count"):
+            assert torch.equal(y[o], want[o]), f"{o} of replay {step}, lengths {n}"
