@@ -431,20 +431,23 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
     if (ts == HILL_OK) ts = from_cuda(counted(launch_score_tc(t, raw, L.score_grid, st), 1));
     if (ts != HILL_OK || raw || part == kScoreStream) return ts;
   }
-  // The tail of a long 16-bit ATTN stream is claimed (score.cu).  Measured,
-  // hill_score, even split / claims (us): 268 MB of keys 42.3 / 46.8, 403 MB
-  // 63.7 / 63.8, 503 MB (40 KV heads) 80.7 / 80.6, 537 MB 83.0 / 79.9.  With 16 KV
-  // heads or fewer a warp has one or two boxes of a tile, too little to hide
-  // a claim's round trip (537 MB: 16 heads 89.8 / 91.3, 8 heads 94.8 / 96.8).  Not
-  // in the split step, whose streams follow one another without a gap (four
-  // pipelined layers 219.7 / 222.0 us), nor from the E4M3 shadow, whose stages are
-  // bound by the warps' own work (111.2 / 117.2).
+  // The tail of a long 16-bit ATTN stream is claimed (score.cu), where the
+  // sequences hold kClaimBytes of keys; a cache that cannot hold them is scored
+  // by the kernel without claims.  Measured, hill_score, even split / claims
+  // (us): 268 MB of keys 42.3 / 46.8, 403 MB 63.7 / 63.8, 537 MB 83.0 / 79.9.
+  // With 16 KV heads or fewer a warp has one or two boxes of a tile, too little
+  // to hide a claim's round trip (537 MB: 16 heads 89.8 / 91.3, 8 heads 94.8 /
+  // 96.8).  Not in the split step, whose streams follow one another without a
+  // gap (four pipelined layers 219.7 / 222.0 us), nor from the E4M3 shadow, whose
+  // stages are bound by the warps' own work (111.2 / 117.2).
   const int64_t stream = (int64_t)d->batch * d->capacity * d->num_kv_heads * 2 * kHeadDim;
   const bool claims = claim && part == kScoreAll && !f8 && G <= 8 && d->num_kv_heads <= score_max_kv_heads() &&
                       d->num_kv_heads > 2 * score_warps() && stream >= kClaimBytes;
   if (claims) {
     a.claim = claim;
     a.claim_tag = next_claim_tag();
+    const int64_t tile_bytes = (int64_t)d->num_kv_heads * score_tile_tokens() * 2 * kHeadDim;
+    a.claim_min = (int)((kClaimBytes + tile_bytes - 1) / tile_bytes);
   }
   hill_status s = part == kScoreNormalise || tc ? HILL_OK : head_passes(d, true, [&](int goff, int nkv, int hoff,
                                                                                       int Gn, bool first) {
@@ -474,7 +477,7 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   f.nslot = (int)L.nslot;
   f.spc = L.score_spc;
   f.score_grid = L.score_grid;
-  f.claims = claims ? 1 : 0;
+  f.claim_min = a.claim_min;
   f.claim = claims ? claim : nullptr;
   f.scores = scores;
   f.accum = accum;

@@ -36,6 +36,7 @@ struct ScoreArgs {
   int nslot;          // partial slots per (b, h): one per work unit (and warp share) that meets b
   ClaimCounter* claim;   // ATTN: [score_warps()] counters of claims, or NULL: even split
   unsigned long long claim_tag;   // of this launch (odd)
+  int claim_min;      // tiles in all from which the tail is claimed
   int kvh;            // RAW with per-KV-head selection: scores/accum [B][Hkv][cap], summed over each group only
   // Query heads per KV head in the data (Gs), the first one this launch
   // handles (hoff) and how many (Gn, at most the kernel's template group G,
@@ -58,7 +59,7 @@ struct FinalizeArgs {
   int B, H, cap, nslot;
   int spc;            // partial slots per scoring unit
   int score_grid;     // CTAs of the scoring launch
-  int claims;         // 1: its tail was claimed tile by tile (Units)
+  int claim_min;      // its claim_min, 0: no claims (Units)
   ClaimCounter* claim;   // the counters, closed here
   float* scores;      // may be NULL when accum is given
   float* accum;       // may be NULL

@@ -50,6 +50,7 @@ constexpr int kBoxBytes = kT * 128;         // one 64-dim half of a tile: 32 swi
 constexpr int kKBytes = 2 * kBoxBytes;
 
 constexpr int kShare16 = 13;   // sixteenths of the tiles dealt out in even shares when the rest is claimed
+constexpr int kMinShare = 5;   // and the least tiles of such a share: more than a warp's first stages reach
 constexpr int kFifo = 8;   // claimed tiles a warp can have in flight: at most kSW + 1
 
 template <int G, bool F8>
@@ -98,13 +99,19 @@ __device__ __forceinline__ int find_seq(const int* tstart, int B, int item) {
 // out and the rest claimed tile by tile: the whole step on 4 x 16-32K tokens
 // 178.8 -> 167.9 us, on 8 x 64K 887.9 -> 860.0 (11/16 and 12/16 the same within
 // 1 %, 14/16 2 % slower).  Opening the counters and a flush of the statistics
-// per claim cost 3-5 us, so short streams keep the even split (run_score).
+// per claim cost 3-5 us, so short streams keep the even split: claim_min is the
+// number of tiles from which the rest is claimed (0: never; run_score).  The
+// tiles counted are those of the lengths at hand, not of the cache's capacity:
+// hill_score on 8 x 1000 tokens in a cache for 8 x 8K takes 14.1 us with the even
+// split and 23.2 with claims, on 16 x 200 in one for 16 x 4K 10.1 and 18.1.
 struct Units {
-  int per, dyn0, grid;   // items of a share; the first item claimed (INT_MAX: none)
-  __device__ __forceinline__ Units(int n_items, int grid_, bool claims) {
+  int per, dyn0, grid;   // items of a share; the first item claimed (n_items: none)
+  __device__ __forceinline__ Units(int n_items, int grid_, int claim_min) {
     grid = grid_;
-    per = claims ? n_items / 16 * kShare16 / grid : (n_items + grid - 1) / grid;
-    dyn0 = claims ? grid * per : 0x7fffffff;
+    const int share = n_items / 16 * kShare16 / grid;
+    const bool claims = claim_min > 0 && n_items >= claim_min && share >= kMinShare;
+    per = claims ? share : (n_items + grid - 1) / grid;
+    dyn0 = claims ? grid * per : n_items;
   }
   __device__ __forceinline__ int of(int item) const { return item < dyn0 ? item / per : grid + (item - dyn0); }
 };
@@ -211,8 +218,9 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
   __syncthreads();
   const int n_items = tstart[B];
   static_assert(!CLAIM || (!RAW && !DEAL && !F8), "tiles are claimed on the 16-bit ATTN stream");
-  const Units units(n_items, gridDim.x, CLAIM);
+  const Units units(n_items, gridDim.x, CLAIM ? a.claim_min : 0);
   const int per = units.per;
+  const bool claims = CLAIM && units.dyn0 < n_items;   // (every CTA then has a share)
   const int it_lo = min(n_items, (int)blockIdx.x * per), it_hi = min(n_items, it_lo + per);   // this CTA's share
   // The warps' shares.  Without DEAL (W = 1) the KV heads are dealt to the
   // warps -- warp w takes g0 + r * kNW, r < ng (0 .. kMaxNg) -- and every warp
@@ -257,17 +265,10 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
   int* fifo = reinterpret_cast<int*>(base + Cfg::kOffFifo) + warp * kFifo;
   unsigned claimed = 0, taken = 0;   // claims of the cursor, and of these taken by the consumer
   unsigned ahead = 0;                // lane 0: the claim made ahead
-  bool is_ahead = false, opened = false;
   auto claim_ahead = [&]() {
-    if (!opened) {
-      if (lane == 0) open_claims(a.claim + warp, a.claim_tag, a.err);
-      opened = true;
-    }
     if (lane == 0) ahead = atomicAdd(&a.claim[warp].count, 1u);
-    is_ahead = true;
   };
   auto claim = [&](Cursor& c) {      // c.item = the next claimed tile, or n_items
-    if (!is_ahead) claim_ahead();
     const unsigned u = __shfl_sync(0xffffffffu, ahead, 0);
     c.r = 0;
     if (u >= (unsigned)(n_items - units.dyn0)) {
@@ -280,12 +281,18 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
     ++claimed;
     claim_ahead();
   };
-  // the cursor's next stage: of its item, its share or a claimed tile
-  const int it_end = CLAIM ? n_items : it_hi;   // where the cursor ends
+  // the cursor's next stage: of its item, its share or a claimed tile.  The
+  // first claim is made ahead at the share's last tile, which the prologue's
+  // kSW stages never reach (kMinShare).
+  static_assert(kMinShare > kSW + 1 || !CLAIM, "a share is longer than the ring");
+  const int it_end = claims ? n_items : it_hi;   // where the cursor ends
   auto next_stage = [&](Cursor& c) {
-    if (!CLAIM || c.r + 1 < ng || c.item + 1 < it_hi) {
+    if (!claims || c.r + 1 < ng || c.item + 1 < it_hi) {
       advance(c);
-      if (CLAIM && c.item + 1 == it_hi && c.r == 0) claim_ahead();
+      if (claims && c.item + 1 == it_hi && c.r == 0) {
+        if (lane == 0) open_claims(a.claim + warp, a.claim_tag, a.err);
+        claim_ahead();
+      }
     } else {
       claim(c);
     }
@@ -367,17 +374,8 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
     const int64_t w1 = min(w0 + hper, a.hist0_words);
     for (int64_t w = w0 + threadIdx.x; w < w1; w += kThreads) a.hist0[w] = 0u;
   }
-  if (CLAIM ? n_items == 0 : it_lo >= it_hi) return;
+  if (it_lo >= it_hi) return;
   if constexpr (F8) prologue();
-  if (CLAIM && ng > 0 && pc.item >= it_hi) {   // a share shorter than the ring: go on with claims
-    claim(pc);
-    while (issued < (uint32_t)kSW && pc.item < n_items) {
-      if (lane == 0) issue(pc, is_slot);
-      ++issued;
-      is_slot = is_slot + 1 == (uint32_t)kSW ? 0u : is_slot + 1;
-      next_stage(pc);
-    }
-  }
   mark_if_done();
 
   // fragment coordinates (mma.sync m16n8k16): C row = token lane/4 (+8),
@@ -822,7 +820,7 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
   }
   __syncthreads();
   const int first_item = s_first;
-  const Units units(s_total, a.score_grid, a.claims != 0);
+  const Units units(s_total, a.score_grid, a.claim_min);
   const int items = (len + kT - 1) / kT;
   const int ns = (units.of(first_item + items - 1) - units.of(first_item) + 1) * a.spc;
   pdl_wait();
@@ -984,7 +982,7 @@ __global__ void __launch_bounds__(kStatsWarps * 32) hill_attn_stats_kernel(Final
   int len = a.lens[b];
   len = len < 0 ? 0 : (len > a.cap ? a.cap : len);
   const int items = (len + kT - 1) / kT;
-  const Units units(t, a.score_grid, a.claims != 0);
+  const Units units(t, a.score_grid, a.claim_min);
   const int ns = items == 0 || !live ? 0 : (units.of(f + items - 1) - units.of(f) + 1) * a.spc;
   pdl_wait();
   pdl_launch_dependents();
@@ -1122,7 +1120,7 @@ cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t s
   // SM the second launch costs more than it saves (about 2 us).
   if (two_kernel || (long long)a.B * ((a.cap + kFinThreads - 1) / kFinThreads) > sms) {
     *kernels = 2;
-    const int W = a.claims ? 4 : 1;   // warps per (b, h)
+    const int W = a.claim_min > 0 ? 4 : 1;   // warps per (b, h)
     const dim3 sgrid((a.B * a.H * W + kStatsWarps - 1) / kStatsWarps);
     cudaError_t e = W > 1 ? launch_pdl(hill_attn_stats_kernel<4>, sgrid, dim3(kStatsWarps * 32), 0, st, 0, a)
                           : launch_pdl(hill_attn_stats_kernel<1>, sgrid, dim3(kStatsWarps * 32), 0, st, 0, a);

@@ -81,6 +81,46 @@ def test_group_sums(H_, Hkv):
         assert not scores[b, :, m:].any()
 
 
+def _claims(ws):
+    """The counts of the eight claim counters (tag 0 once closed, count, a pad word) in a workspace that held 0x5A bytes
+    before the call; None where nothing was claimed."""
+    start = -ws.data_ptr() % 256
+    rows = ws[start:start + (ws.numel() - start) // 256 * 256].view(torch.int32).view(-1, 64)
+    filler = 0x5A5A5A5A
+    head = rows[:, :32].view(-1, 8, 4)
+    hit = (head[..., :2] == 0).all(-1).all(-1) & (head[..., 3] == filler).all(-1) & (rows[:, 32:] == filler).all(-1)
+    assert int(hit.sum()) <= 1
+    counts = head[hit][..., 2].flatten().tolist()
+    return counts if counts and filler not in counts else None
+
+
+@pytest.mark.parametrize("lens,claimed", [([8192] * 8, True), ([8192] * 7 + [8160], False), ([1000] * 8, False),
+                                          ([65536] + [0] * 7, True), ([65504] + [0] * 7, False)])
+def test_claims_by_the_tokens_present(lens, claimed):
+    """A cache that could hold more than 512 MB of keys: the tail is claimed where the sequences in it do (65536 tokens
+    of 32 heads), and not where they are short."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_18750_gb300 import build, hill as H
+    build.build()
+    cap = max(9000, max(lens) + 64)
+    K = torch.randn(len(lens), 32, cap, 128, dtype=torch.float16, device="cuda")
+    q = torch.randn(len(lens), 32, 128, dtype=torch.float16, device="cuda")
+    desc = H.make_desc(q, K)
+    assert K.numel() * 2 >= 512 << 20
+    ws = H.alloc_workspace(desc, 0, 0)
+    ws.fill_(0x5A)
+    scores = torch.zeros(len(lens), cap, device="cuda")
+    H.hill_score(desc, q, K, torch.tensor(lens, dtype=torch.int32, device="cuda"), 0, scores, None, ws)
+    H.hill_sync_status()
+    counts = _claims(ws)
+    assert (counts is not None) == claimed
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    tiles = sum((m + 31) // 32 for m in lens)
+    # every warp index claims each tile past the shares once, and then once more per CTA
+    assert not claimed or counts == [tiles - sms * (tiles // 16 * 13 // sms) + sms] * 8
+
+
 @pytest.mark.parametrize("lens", [[7100] * 8, [7100, 0, 1, 31, 32, 33, 4000, 7099], [0, 0, 0, 0, 0, 0, 0, 200],
                                   [5000, 0, 0, 0, 0, 0, 0, 0], [640, 641, 639, 7, 0, 0, 1500, 3]])
 @pytest.mark.parametrize("Hq,Hkv", [(32, 32), (64, 32), (48, 16)])
