@@ -435,6 +435,10 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   // sequences hold kClaimBytes of keys; a cache that cannot hold them is scored
   // by the kernel without claims.  Measured, hill_score, even split / claims
   // (us): 268 MB of keys 42.3 / 46.8, 403 MB 63.7 / 63.8, 537 MB 83.0 / 79.9.
+  // The partials of claimed tiles are many and take the two-kernel
+  // normalisation, so only caches that take it anyway have claims (8 x 8192
+  // tokens do not: full ones would gain 2 us of 80, but sequences of 819 in them
+  // take 12.3 us with one kernel and 13.2 with two).
   // With 16 KV heads or fewer a warp has one or two boxes of a tile, too little
   // to hide a claim's round trip (537 MB: 16 heads 89.8 / 91.3, 8 heads 94.8 /
   // 96.8).  Not in the split step, whose streams follow one another without a
@@ -442,7 +446,8 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   // stages are bound by the warps' own work (111.2 / 117.2).
   const int64_t stream = (int64_t)d->batch * d->capacity * d->num_kv_heads * 2 * kHeadDim;
   const bool claims = claim && part == kScoreAll && !f8 && G <= 8 && d->num_kv_heads <= score_max_kv_heads() &&
-                      d->num_kv_heads > 2 * score_warps() && stream >= kClaimBytes;
+                      d->num_kv_heads > 2 * score_warps() && stream >= kClaimBytes &&
+                      attn_finalize_waves(d->batch, d->capacity, di.sms) > 2;
   if (claims) {
     a.claim = claim;
     a.claim_tag = next_claim_tag();

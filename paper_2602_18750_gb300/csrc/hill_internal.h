@@ -207,6 +207,8 @@ int score_max_kv_heads();
 int score_deal_warps(int nkv, int G);
 cudaError_t launch_score(const ScoreArgs& a, int dtype, int G, bool raw, bool f8, bool deal, int grid,
                          cudaStream_t st);
+// CTAs per SM of the normalisation with one block of tokens each, rounded up.
+int attn_finalize_waves(int B, int cap, int sms);
 // Launches the normalisation (one or two kernels: *kernels is set to the
 // count).  two_kernel: always combine the partials in their own kernel first,
 // so that the finalize kernel takes its small form (at most 64 registers),

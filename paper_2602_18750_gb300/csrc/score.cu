@@ -1101,6 +1101,10 @@ static cudaError_t launch_finalize_t(const FinalizeArgs& a, cudaStream_t st) {
                                 : launch(hill_attn_finalize_kernel<STATS, -1>);
 }
 
+int attn_finalize_waves(int B, int cap, int sms) {
+  return (int)(((int64_t)B * ((cap + kFinThreads - 1) / kFinThreads) + sms - 1) / sms);
+}
+
 cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t st, int* kernels,
                                  bool two_kernel) {
   FinalizeArgs a = a0;
@@ -1113,12 +1117,17 @@ cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t s
     while (a.tpt < kFinMaxTpt &&
            (long long)a.B * ((a.cap + kFinThreads * a.tpt - 1) / (kFinThreads * a.tpt)) > 2LL * sms)
       a.tpt <<= 1;
-  // With more than one CTA per SM the partials are combined once per (b, h)
-  // in a kernel of their own instead of once per CTA: scores to selection at
-  // 4 x 16K tokens of one KV head (304 partials per head) 23.8 against 27.7
-  // us, 4 x 16-32K 142.1 against 142.6, 1 x 128K the same; up to one CTA per
-  // SM the second launch costs more than it saves (about 2 us).
-  if (two_kernel || (long long)a.B * ((a.cap + kFinThreads - 1) / kFinThreads) > sms) {
+  // The partials are combined once per (b, h) in a kernel of their own instead
+  // of once per CTA with more than two CTAs per SM (attn_finalize_waves), and
+  // with more than one where a head has more partials than a warp holds in
+  // registers.  Measured, hill_score, one / two kernels (us): 4 x 10K tokens, 8
+  // KV heads (38 partials a head) 18.5 / 19.8, with 1000 tokens in each 6.9 / 6.9
+  // and issued eagerly 11.0 / 12.7; 8 x 6000, 32 KV heads 60.1 / 60.0, with 600 in
+  // each 9.8 / 10.3; 1 x 64K, 8 KV heads (152 partials) 25.6 / 26.0; 16 x 4K of
+  // one KV head (76) 16.6 / 18.0, but 4 x 16K of one (304), scores to selection,
+  // 27.7 / 23.8.
+  if (two_kernel || attn_finalize_waves(a.B, a.cap, sms) > 2 ||
+      (attn_finalize_waves(a.B, a.cap, sms) > 1 && a.score_grid * a.spc / a.B > 32 * kFinU)) {
     *kernels = 2;
     const int W = a.claim_min > 0 ? 4 : 1;   // warps per (b, h)
     const dim3 sgrid((a.B * a.H * W + kStatsWarps - 1) / kStatsWarps);

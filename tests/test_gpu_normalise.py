@@ -94,6 +94,38 @@ def _claims(ws):
     return counts if counts and filler not in counts else None
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,n,launches", [
+    (4, 32, 8, 10000, 2), (1, 32, 8, 65536, 2), (16, 32, 1, 4096, 2), (8, 32, 32, 8192, 2),   # up to two blocks per SM
+    (4, 32, 1, 16384, 3),                       # with more partials per head than a warp's registers hold
+    (1, 32, 8, 80000, 3), (1, 32, 32, 80000, 3),
+])
+def test_launches_of_the_normalisation(B, Hq, Hkv, n, launches):
+    """Which sizes combine the partials in a kernel of their own (152 SMs), and the scores of both forms at the sizes
+    where they meet, in a cache that is filled and in one that is nearly empty."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("sizes of 152 SMs")
+    from paper_2602_18750_gb300 import build, hill as H
+    build.build()
+    g = torch.Generator(device="cuda").manual_seed(n + Hkv)
+    K = torch.randn(B, Hkv, n, 128, generator=g, device="cuda").half()
+    q = (2 * torch.randn(B, Hq, 128, generator=g, device="cuda")).half()
+    desc = H.make_desc(q, K)
+    ws = H.alloc_workspace(desc, 0, 0)
+    ws.fill_(0xFF)
+    for m in (n, n // 10):
+        scores = torch.zeros(B, n, device="cuda")
+        before = H.hill_kernel_launches()
+        H.hill_score(desc, q, K, torch.full((B,), m, dtype=torch.int32, device="cuda"), 0, scores, None, ws)
+        assert H.hill_kernel_launches() - before == launches
+        H.hill_sync_status()
+        for b in (0, B - 1):
+            z = torch.stack([K[b, h * Hkv // Hq, :m].double() @ q[b, h].double() for h in range(Hq)]) / np.sqrt(128)
+            ref = torch.softmax(z, -1).sum(0)
+            assert torch.all((scores[b, :m].double() - ref).abs() <= 2e-5 * ref)
+
+
 @pytest.mark.parametrize("lens,claimed", [([8192] * 8, True), ([8192] * 7 + [8160], False), ([1000] * 8, False),
                                           ([65536] + [0] * 7, True), ([65504] + [0] * 7, False)])
 def test_claims_by_the_tokens_present(lens, claimed):
@@ -103,7 +135,7 @@ def test_claims_by_the_tokens_present(lens, claimed):
         pytest.skip("no CUDA device")
     from paper_2602_18750_gb300 import build, hill as H
     build.build()
-    cap = max(9000, max(lens) + 64)
+    cap = max(10000, max(lens) + 64)   # (more than two blocks of tokens per SM)
     K = torch.randn(len(lens), 32, cap, 128, dtype=torch.float16, device="cuda")
     q = torch.randn(len(lens), 32, 128, dtype=torch.float16, device="cuda")
     desc = H.make_desc(q, K)
