@@ -210,7 +210,7 @@ struct Layout {
   size_t scores, logits, partials, stats, hist0, attn_part, q8, sq, total;
   bool has_hist0;
   size_t claim;      // claim counters of the scoring kernel
-  bool has_claim;
+  int claim_min;     // tiles from which its tail is claimed (0: never)
   int64_t nslot;     // ATTN partial slots per (b, h)
   int score_grid, attn_grid, splits;
   int score_spc;   // ATTN partial slots per scoring CTA
@@ -232,6 +232,31 @@ int score_grid_for(const hill_desc* d, int sms, bool split_grid = false) {
   return g < 1 ? 1 : (int)g;
 }
 
+// The tail of a long 16-bit ATTN stream is claimed (score.cu), where the
+// sequences hold kClaimBytes of keys; a cache that cannot hold them is scored
+// by the kernel without claims.  Measured, hill_score, even split / claims
+// (us): 268 MB of keys 42.3 / 46.8, 403 MB 63.7 / 63.8, 537 MB 83.0 / 79.9.
+// The partials of claimed tiles are many and take the two-kernel
+// normalisation, so only caches that take it anyway have claims (8 x 8192
+// tokens do not: full ones would gain 2 us of 80, but sequences of 819 in them
+// take 12.3 us with one kernel and 13.2 with two).
+// With 16 KV heads or fewer a warp has one or two boxes of a tile, too little
+// to hide a claim's round trip (537 MB: 16 heads 89.8 / 91.3, 8 heads 94.8 /
+// 96.8).  Not in the split step, whose streams follow one another without a
+// gap (four pipelined layers 219.7 / 222.0 us), nor from the E4M3 shadow, whose
+// stages are bound by the warps' own work (111.2 / 117.2).
+constexpr int64_t kClaimBytes = (int64_t)512 << 20;
+
+// The tiles from which a call of this layout claims; 0: it never does.
+int claim_min_for(const hill_desc* d, int mode, int sms) {
+  const int64_t tile_bytes = (int64_t)d->num_kv_heads * score_tile_tokens() * 2 * kHeadDim;
+  if (mode != HILL_SCORE_ATTN || d->num_kv_heads <= 2 * score_warps() || d->num_kv_heads > score_max_kv_heads() ||
+      d->num_q_heads / d->num_kv_heads > 8 || attn_finalize_waves(d->batch, d->capacity, sms) <= 2 ||
+      (int64_t)d->batch * d->capacity * (tile_bytes / score_tile_tokens()) < kClaimBytes)
+    return 0;
+  return (int)((kClaimBytes + tile_bytes - 1) / tile_bytes);
+}
+
 // Workspace regions of a call.  score_only: hill_score and its variants,
 // which write the caller's scores and run no selection or attention, need
 // only the ATTN normalisation's logits, partials and statistics.  e4m3_query:
@@ -248,12 +273,11 @@ Layout layout_for(const hill_desc* d, int mode, int max_k, int sms, bool score_o
   L.score_spc = d->num_kv_heads > score_max_kv_heads()
                     ? 1
                     : score_deal_warps(d->num_kv_heads, d->num_q_heads / d->num_kv_heads);
-  // the tail of a long K stream is claimed tile by tile (run_score); the
-  // allocation-free entry point keeps the even split and its documented scratch
-  L.has_claim = mode == HILL_SCORE_ATTN && e4m3_query && L.score_spc == 1 && !split_grid;
+  // the allocation-free entry point keeps the even split and its documented scratch
+  L.claim_min = e4m3_query && !split_grid ? claim_min_for(d, mode, sms) : 0;
   // (every unit that meets a sequence holds one of its tiles)
   const int64_t tiles = std::max(1, (d->capacity + score_tile_tokens() - 1) / score_tile_tokens());
-  const int64_t units = L.has_claim ? score_claim_slots(d->batch * tiles, L.score_grid) : L.score_grid;
+  const int64_t units = L.claim_min > 0 ? score_claim_slots(d->batch * tiles, L.score_grid) : L.score_grid;
   L.nslot = (e4m3_query ? std::min(tiles, units) : units) * L.score_spc;
   L.attn_grid = sms;
   L.splits = score_only ? 0 : attn_max_segments(max_k < 0 ? 0 : max_k);
@@ -275,7 +299,7 @@ Layout layout_for(const hill_desc* d, int mode, int max_k, int sms, bool score_o
   L.has_hist0 = mode == HILL_SCORE_ATTN && max_k > 0 && !score_only;
   if (L.has_hist0) off += align_up(B * (size_t)select_hist_bins() * sizeof(uint32_t));
   L.claim = off;
-  if (L.has_claim) off += align_up(score_warps() * sizeof(ClaimCounter));
+  if (L.claim_min > 0) off += align_up(score_warps() * sizeof(ClaimCounter));
   L.attn_part = off;
   off += align_up(B * H * (size_t)L.splits * (2 + kHeadDim) * sizeof(float));
   // E4M3 query codes [B][Hkv][16][128] and scales [B][H]
@@ -327,9 +351,6 @@ hill_status head_passes(const hill_desc* d, bool kv_split, F&& f, int per_pass =
 // stream only (the scoring kernel), or the ATTN normalisation only.
 constexpr int kScoreAll = 0, kScoreStream = 1, kScoreNormalise = 2;
 
-// Key bytes from which the scoring kernel's tail is claimed (run_score).
-constexpr int64_t kClaimBytes = (int64_t)512 << 20;
-
 hill_status run_score(const hill_desc* d, const void* q, const void* k, const int32_t* lens, int mode,
                       float* scores, float* accum, unsigned char* base, const Layout& L,
                       const DeviceInfo& di, cudaStream_t st, uint32_t* hist0 = nullptr, int recent = 0,
@@ -379,7 +400,6 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   // or above the pass's heads (8 for the dealing kernel)
   const bool deal = L.score_spc > 1;
   a.Gs = G;
-  ClaimCounter* claim = L.has_claim ? reinterpret_cast<ClaimCounter*>(base + L.claim) : nullptr;
   // E4M3 scoring on the tensor cores' native 8-bit path (score_tc.cu) for
   // per-sequence importance with 2 to 16 query heads per KV head (at most
   // score_tc_max_heads() in all, one pass over the KV heads) and at least
@@ -431,28 +451,12 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
     if (ts == HILL_OK) ts = from_cuda(counted(launch_score_tc(t, raw, L.score_grid, st), 1));
     if (ts != HILL_OK || raw || part == kScoreStream) return ts;
   }
-  // The tail of a long 16-bit ATTN stream is claimed (score.cu), where the
-  // sequences hold kClaimBytes of keys; a cache that cannot hold them is scored
-  // by the kernel without claims.  Measured, hill_score, even split / claims
-  // (us): 268 MB of keys 42.3 / 46.8, 403 MB 63.7 / 63.8, 537 MB 83.0 / 79.9.
-  // The partials of claimed tiles are many and take the two-kernel
-  // normalisation, so only caches that take it anyway have claims (8 x 8192
-  // tokens do not: full ones would gain 2 us of 80, but sequences of 819 in them
-  // take 12.3 us with one kernel and 13.2 with two).
-  // With 16 KV heads or fewer a warp has one or two boxes of a tile, too little
-  // to hide a claim's round trip (537 MB: 16 heads 89.8 / 91.3, 8 heads 94.8 /
-  // 96.8).  Not in the split step, whose streams follow one another without a
-  // gap (four pipelined layers 219.7 / 222.0 us), nor from the E4M3 shadow, whose
-  // stages are bound by the warps' own work (111.2 / 117.2).
-  const int64_t stream = (int64_t)d->batch * d->capacity * d->num_kv_heads * 2 * kHeadDim;
-  const bool claims = claim && part == kScoreAll && !f8 && G <= 8 && d->num_kv_heads <= score_max_kv_heads() &&
-                      d->num_kv_heads > 2 * score_warps() && stream >= kClaimBytes &&
-                      attn_finalize_waves(d->batch, d->capacity, di.sms) > 2;
+  // (the split step's layouts have no claims, and the E4M3 shadow makes none)
+  const bool claims = L.claim_min > 0 && !f8;
   if (claims) {
-    a.claim = claim;
+    a.claim = reinterpret_cast<ClaimCounter*>(base + L.claim);
     a.claim_tag = next_claim_tag();
-    const int64_t tile_bytes = (int64_t)d->num_kv_heads * score_tile_tokens() * 2 * kHeadDim;
-    a.claim_min = (int)((kClaimBytes + tile_bytes - 1) / tile_bytes);
+    a.claim_min = L.claim_min;
   }
   hill_status s = part == kScoreNormalise || tc ? HILL_OK : head_passes(d, true, [&](int goff, int nkv, int hoff,
                                                                                       int Gn, bool first) {
@@ -483,7 +487,7 @@ hill_status run_score(const hill_desc* d, const void* q, const void* k, const in
   f.spc = L.score_spc;
   f.score_grid = L.score_grid;
   f.claim_min = a.claim_min;
-  f.claim = claims ? claim : nullptr;
+  f.claim = a.claim;
   f.scores = scores;
   f.accum = accum;
   f.hist0 = hist0;

@@ -153,6 +153,26 @@ def test_claims_by_the_tokens_present(lens, claimed):
     assert not claimed or counts == [tiles - sms * (tiles // 16 * 13 // sms) + sms] * 8
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,cap,claims", [(1, 32, 8, 131072, False), (4, 32, 16, 32768, False), (4, 40, 40, 32768, False),
+                                                 (4, 32, 32, 12000, False), (4, 32, 1, 16384, False), (4, 32, 32, 32768, True)])
+def test_workspace_without_claims(B, Hq, Hkv, cap, claims):
+    """A layout that never claims holds one partial slot per scoring CTA (and warp share), as hill_score_noalloc
+    documents it; one that may claim holds more."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_18750_gb300 import build, hill as H
+    build.build()
+    K = torch.zeros(1, 1, 1, 128, dtype=torch.float16, device="cuda").expand(B, Hkv, cap, 128)
+    desc = H.make_desc(torch.zeros(B, Hq, 128, dtype=torch.float16, device="cuda"), K)
+    attn = H.hill_workspace_bytes(desc, 0, 0) - H.hill_workspace_bytes(desc, 1, 0)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    warps = 8 // Hkv if Hkv <= 4 and Hq // Hkv >= 5 else 1
+    up = lambda n: (n + 255) // 256 * 256  # noqa: E731
+    tiles = (cap + 31) // 32
+    bound = up(4 * B * Hq * tiles * 32) + up(8 * B * Hq * min(sms, B * tiles) * warps) + up(8 * B * Hq)
+    assert (attn > bound) == claims
+
+
 @pytest.mark.parametrize("lens", [[7100] * 8, [7100, 0, 1, 31, 32, 33, 4000, 7099], [0, 0, 0, 0, 0, 0, 0, 200],
                                   [5000, 0, 0, 0, 0, 0, 0, 0], [640, 641, 639, 7, 0, 0, 1500, 3]])
 @pytest.mark.parametrize("Hq,Hkv", [(32, 32), (64, 32), (48, 16)])
