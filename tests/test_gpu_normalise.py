@@ -173,26 +173,33 @@ def test_workspace_without_claims(B, Hq, Hkv, cap, claims):
     assert (attn > bound) == claims
 
 
-@pytest.mark.parametrize("lens", [[7100] * 8, [7100, 0, 1, 31, 32, 33, 4000, 7099], [0, 0, 0, 0, 0, 0, 0, 200],
-                                  [5000, 0, 0, 0, 0, 0, 0, 0], [640, 641, 639, 7, 0, 0, 1500, 3]])
-@pytest.mark.parametrize("Hq,Hkv", [(32, 32), (64, 32), (48, 16)])
-def test_claimed_tail_of_a_large_cache(Hq, Hkv, lens):
-    """A cache large enough for the scoring kernel's tail to be claimed, full, ragged and nearly empty (shares shorter
-    than a warp's ring, no share at all): right against float64 and the same bits every time."""
+@pytest.mark.parametrize("lens,claimed", [
+    ([8200] * 8, True), ([30000, 0, 1, 20000, 641, 16000, 33, 100], True), ([65537] + [0] * 7, True),
+    ([0] * 7 + [66000], True), ([0, 31, 32, 33, 66000, 0, 7, 1], True), ([640, 641, 639, 7, 0, 0, 1500, 3], False),
+])
+@pytest.mark.parametrize("Hq,Hkv,dtype", [(32, 32, torch.float16), (64, 32, torch.bfloat16), (96, 32, torch.bfloat16),
+                                          (24, 24, torch.bfloat16), (40, 20, torch.float16), (136, 17, torch.bfloat16)])
+def test_claimed_tail_of_a_large_cache(Hq, Hkv, dtype, lens, claimed):
+    """A cache large enough for the scoring kernel's tail to be claimed, full, ragged, with empty sequences anywhere and
+    nearly empty; groups of 1 to 8, uneven heads per warp: right against float64, the same bits every time and in the
+    fused step, and the workspace's counters say that tiles were claimed (from 512 MB of keys on: lengths are given for
+    32 KV heads)."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2602_18750_gb300 import build, hill as H
     build.build()
-    B, cap, G = 8, 7168 * 32 // Hkv, Hq // Hkv
+    lens = [-(-m * 32 // Hkv) for m in lens]
+    B, G, cap = 8, Hq // Hkv, max(max(lens), 10000 * 32 // Hkv)
     g = torch.Generator(device="cuda").manual_seed(sum(lens) + Hq)
-    K = torch.empty(B, Hkv, cap, 128, dtype=torch.bfloat16, device="cuda")
+    K = torch.empty(B, Hkv, cap, 128, dtype=dtype, device="cuda")
     for b, m in enumerate(lens):
-        K[b, :, :m] = torch.randn(Hkv, m, 128, generator=g, device="cuda").bfloat16()
+        K[b, :, :m] = torch.randn(Hkv, m, 128, generator=g, device="cuda").to(dtype)
         K[b, :, m:] = float("nan")
-    q = (2 * torch.randn(B, Hq, 128, generator=g, device="cuda")).bfloat16()
+    q = (2 * torch.randn(B, Hq, 128, generator=g, device="cuda")).to(dtype)
     desc = H.make_desc(q, K)
     lens_t = torch.tensor(lens, dtype=torch.int32, device="cuda")
-    ws = H.alloc_workspace(desc, 0, 0)
+    kept = torch.tensor([min(m, 50) for m in lens], dtype=torch.int32, device="cuda")
+    ws = H.alloc_workspace(desc, 0, 50)
     first = None
     for fill in (0, 0xFF, 0x5A):
         ws.fill_(fill)
@@ -201,11 +208,22 @@ def test_claimed_tail_of_a_large_cache(Hq, Hkv, lens):
         H.hill_sync_status()
         assert first is None or torch.equal(scores, first)
         first = scores
+    assert (_claims(ws) is not None) == claimed
+    accum, scores = torch.zeros(B, cap, device="cuda"), torch.zeros(B, cap, device="cuda")
+    idx = torch.zeros(B, 50, dtype=torch.int32, device="cuda")
+    H.hill_evict_step(desc, q, K, None, lens_t, kept, 50, 0, accum, scores, idx, torch.empty_like(kept), None, ws)
+    H.hill_sync_status()
+    assert torch.equal(scores, first) and torch.equal(accum, first)
     for b, m in enumerate(lens):
-        z = torch.stack([K[b, h // G, :m].double() @ q[b, h].double() for h in range(Hq)]) / np.sqrt(128)
-        ref = torch.softmax(z, -1).sum(0)
-        assert m == 0 or torch.all((scores[b, :m].double() - ref).abs() <= 2e-5 * ref)
         assert not scores[b, m:].any()
+        if m == 0:
+            continue
+        ref = torch.zeros(m, dtype=torch.float64, device="cuda")
+        for h in range(Hq):
+            ref += torch.softmax(K[b, h // G, :m].double() @ q[b, h].double() / np.sqrt(128), -1)
+        assert torch.all((scores[b, :m].double() - ref).abs() <= 2e-5 * ref)
+        order = torch.sort(scores[b, :m], descending=True, stable=True).indices[:min(m, 50)]
+        assert torch.equal(idx[b, :min(m, 50)].long(), order.sort().values)
 
 
 @pytest.mark.parametrize("Hq,Hkv,cap", [(32, 32, 24000), (48, 24, 32000)])
