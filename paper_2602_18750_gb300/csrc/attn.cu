@@ -722,7 +722,9 @@ cudaError_t launch_attn_cl(const AttnArgs& a, int sms, cudaStream_t st, bool* do
   cudaError_t e = triples <= sms ? attn_cluster_size<DT, G, kAW>(triples, nb, sms, &c8, &r8) : cudaSuccess;
   if (e == cudaSuccess) e = attn_cluster_size<DT, G, kAW / 2>(triples, nb, sms, &c4, &r4);
   if (e != cudaSuccess) return e;
-  const bool half = c8 == 0 || (c4 > 0 && r4 < r8);
+  // CTAs of 4 warps, which spread a (b, g) over twice as many SMs, unless they
+  // take more rounds
+  const bool half = c8 == 0 || (c4 > 0 && r4 <= r8);
   const int C = half ? c4 : c8, rounds = half ? r4 : r8;
   const int64_t even = (triples * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
   // A round (one more batch per warp) costs about 1.6 us where latency bounds
@@ -736,6 +738,17 @@ cudaError_t launch_attn_cl(const AttnArgs& a, int sms, cudaStream_t st, bool* do
   // 64K 24.7 / 18.7 (1 / 7), k 30 % of 128K 32.4 / 41.5 (3 / 20).
   const int64_t passes = (a.Gs + 15) / 16;
   if (C == 0 || even > 32 || rounds > even + even / 4 + 3 * passes) return cudaSuccess;
+  // The counts are not known here.  With one sequence at max_k and the others
+  // nearly empty the even split has only that one's batches to deal out
+  // (`one` rounds), while its clusters still take all their rounds, at about 1
+  // us each.  Measured, even split / clusters, equal counts and one long one (us,
+  // rounds - one in brackets): 32 heads, 8 x 819 18.8 / 14.9, [819, 7 x 50] 10.3 /
+  // 10.2 (6); 8 KV heads, 16 x 1638 23.4 / 15.9, 11.0 / 11.4 (6); 4 x 6553 19.7 /
+  // 16.0, 12.0 / 11.9 (5); but 32 heads, 4 x 2457 31.8 / 28.4 and [3277, 3 x 200]
+  // 13.8 / 17.6 (10); 40 heads, 6 x 1500 35.5 / 31.4, [1500, 5 x 50] 10.4 / 15.5 (10)
+  const int units = a.kvh ? a.B * a.Hkv : a.B;
+  const int64_t one = (triples / units * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
+  if (units > 1 && rounds > one + 6 * passes) return cudaSuccess;
   *done = true;
   const dim3 grid((unsigned)(triples * C));
   return half ? launch_pdl(hill_sparse_attn_kernel<DT, G, true, kAW / 2>, grid, dim3(kAThreads / 2), AttnCfg::smem(kAW / 2),

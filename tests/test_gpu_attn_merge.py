@@ -72,3 +72,41 @@ def test_attention_over_every_split(H, case, dtype):
             assert torch.equal(out, first), "the merge order must not depend on which CTA arrives last"
         first = out.clone()
         out.fill_(float("nan"))
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,n,kept,max_k,launches", [
+    (8, 32, 32, 4096, [819] * 8, 819, 1), (8, 32, 32, 4096, [819] + [0] * 7, 819, 1),
+    (4, 32, 32, 4096, [3277, 200, 0, 200], 3277, 2),    # one long sequence: its batches over all warps
+    (6, 40, 40, 2048, [1500, 50, 50, 0, 50, 1], 1500, 2),
+    (1, 32, 32, 4096, [3277], 3277, 1), (2, 32, 32, 4096, [3277, 1], 3277, 1),
+    (16, 32, 1, 7000, [6400] + [50] * 15, 6400, 1),     # two passes over the heads
+    (4, 32, 8, 4096, [100] * 4, 4000, 1),               # an index width far above the counts
+])
+def test_form_by_index_width(H, B, Hq, Hkv, n, kept, max_k, launches):
+    """Which widths take clusters per (sequence, KV head) (one launch) and which the even split and its merge (152 SMs):
+    where the counts may differ, a single long sequence must not be left to a few CTAs."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("sizes of 152 SMs")
+    g = torch.Generator(device="cuda").manual_seed(max_k + B)
+    K, V = (torch.randn(B, Hkv, n, 128, generator=g, device="cuda").half() for _ in range(2))
+    q = torch.randn(B, Hq, 128, generator=g, device="cuda").half()
+    desc = H.make_desc(q, K, V)
+    idx = torch.full((B, max_k), -1, dtype=torch.int32, device="cuda")
+    for b, m in enumerate(kept):
+        idx[b, :m] = torch.randperm(n, generator=g, device="cuda")[:m].sort().values.int()
+    count = torch.tensor(kept, dtype=torch.int32, device="cuda")
+    out = torch.full((B, Hq, 128), float("nan"), device="cuda")
+    ws = H.alloc_workspace(desc, 0, max_k)
+    ws.fill_(0xFF)
+    before = H.hill_kernel_launches()
+    H.hill_gather_sparse_attn(desc, q, K, V, idx, count, max_k, out, ws)
+    assert H.hill_kernel_launches() - before == launches
+    H.hill_sync_status()
+    ref = torch.zeros(B, Hq, 128, dtype=torch.float64, device="cuda")
+    for b, m in enumerate(kept):
+        t = idx[b, :m].long()
+        for h in range(Hq if m else 0):
+            g_ = h * Hkv // Hq
+            p = torch.softmax(K[b, g_, t].double() @ q[b, h].double() / math.sqrt(128), 0)
+            ref[b, h] = p @ V[b, g_, t].double()
+    check_attn(out.cpu().numpy(), ref.cpu().numpy())
