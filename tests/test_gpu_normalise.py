@@ -81,10 +81,11 @@ def test_group_sums(H_, Hkv):
         assert not scores[b, :, m:].any()
 
 
-def _claims(ws):
+def _claims(ws, desc):
     """The counts of the eight claim counters (tag 0 once closed, count, a pad word) in a workspace that held 0x5A bytes
-    before the call; None where nothing was claimed."""
-    start = -ws.data_ptr() % 256
+    before a hill_score call; None where nothing was claimed. The logits, which come first, are skipped: their lines are
+    discarded from L2 and may read as anything."""
+    start = -ws.data_ptr() % 256 + (4 * desc.batch * desc.num_q_heads * (-(-desc.capacity // 32) * 32) + 255) // 256 * 256
     rows = ws[start:start + (ws.numel() - start) // 256 * 256].view(torch.int32).view(-1, 64)
     filler = 0x5A5A5A5A
     head = rows[:, :32].view(-1, 8, 4)
@@ -145,7 +146,7 @@ def test_claims_by_the_tokens_present(lens, claimed):
     scores = torch.zeros(len(lens), cap, device="cuda")
     H.hill_score(desc, q, K, torch.tensor(lens, dtype=torch.int32, device="cuda"), 0, scores, None, ws)
     H.hill_sync_status()
-    counts = _claims(ws)
+    counts = _claims(ws, desc)
     assert (counts is not None) == claimed
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     tiles = sum((m + 31) // 32 for m in lens)
@@ -208,7 +209,7 @@ def test_claimed_tail_of_a_large_cache(Hq, Hkv, dtype, lens, claimed):
         H.hill_sync_status()
         assert first is None or torch.equal(scores, first)
         first = scores
-    assert (_claims(ws) is not None) == claimed
+    assert (_claims(ws, desc) is not None) == claimed
     accum, scores = torch.zeros(B, cap, device="cuda"), torch.zeros(B, cap, device="cuda")
     idx = torch.zeros(B, 50, dtype=torch.int32, device="cuda")
     H.hill_evict_step(desc, q, K, None, lens_t, kept, 50, 0, accum, scores, idx, torch.empty_like(kept), None, ws)
