@@ -121,6 +121,7 @@ struct SelectArgs {
   const int32_t* k;
   int B, cap, max_k;
   int lcap, list_words, pad_shift;   // crossing-bin list entries per CTA, words of the list, spare quads of the keys (set by the launcher)
+  int alone_max;      // ranked tokens (and places before the first) up to which a cluster's first CTA works alone (set by the launcher)
   const uint32_t* hist0;   // optional [B][2048]: counts of the leading 11-bit key digit (tokens j < len - recent)
   int rows_per_seq;   // key rows per sequence: 1, or Hkv with per-KV-head selection (row r reads lens/k of r / rows_per_seq)
   int recent;         // BKP: the most recent min(recent, len) tokens are kept outright (0: none)

@@ -56,7 +56,11 @@ constexpr int kKeysMax = 48128;    // keys per CTA that fit shared memory beside
 constexpr int kSelSmem = 225 * 1024;   // dynamic; 1.4 KB static beside it
 constexpr int kChunk = 4608;         // keys per CTA that a row is spread to, SMs permitting
 constexpr int kChunkMax = 16384;     // and at most, while the cluster can grow
-constexpr int kFew = 256;          // listed keys that are ranked directly
+constexpr int kAlone = 8192;       // ranked tokens up to which one CTA is faster than a cluster
+// Listed keys that are ranked directly: 64 of them take as long as a histogram
+// and its search, 200 take 1.5 us more (a row of 4000 keys with 5 % kept 4.7 us,
+// with up to 256 ranked 5.6).
+constexpr int kFew = 64;
 constexpr int kListMax = 8192;     // crossing-bin keys of a row held by every CTA
 
 // The bin in which the running count from the top bin down reaches `need`,
@@ -160,7 +164,17 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
     kk = min(kk, a.max_k - win);
   }
   const bool search = kk > 0 && kk < older;   // the same in every CTA of the row
-  if (CL) {
+  const float* row_key = a.key + (int64_t)row * a.cap;
+  const int s0 = (int)((reinterpret_cast<uintptr_t>(row_key) >> 2) & 3u);
+  // A short row of a large cache is searched by the cluster's first CTA alone,
+  // without the exchanges.  4 rows in a cache of 16K, four CTAs each / alone
+  // (us): 1000 tokens 6.4 / 4.6, 4000 7.5 / 5.2, 6000 6.7 / 5.7, 8000 6.9 / 6.0.
+  const bool alone = CL && older + s0 <= a.alone_max;
+  const bool multi = CL && !alone;   // the CTAs search together
+  const int S = alone ? 1 : C, rs = alone ? 0 : r;   // the CTAs that search; this one among them
+  const bool mine_to_search = search && (!alone || r == 0);
+  const int lcap = alone ? C * a.lcap : a.lcap;
+  if (multi) {
     if (search) cluster.barrier_arrive();   // A: every CTA has started and cleared its memory
   } else {
     __syncthreads();
@@ -171,29 +185,27 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
   // CTA's quads are read from global memory in order and kept in shared
   // memory, from where thread t takes the q quads t * q .. t * q + q - 1; a
   // spare quad in every eight keeps both sides free of bank conflicts.
-  const float* row_key = a.key + (int64_t)row * a.cap;
-  const int s0 = (int)((reinterpret_cast<uintptr_t>(row_key) >> 2) & 3u);
-  const int share = (((older + s0 + C - 1) / C) + 3) & ~3;
+  const int share = (((older + s0 + S - 1) / S) + 3) & ~3;
   const int nq = share / 4, q = (nq + T - 1) / T;
-  const int jc = r * share - s0;    // the CTA's first token (maybe negative: none there)
+  const int jc = rs * share - s0;   // the CTA's first token (maybe negative: none there)
   const int hi = min(older, jc + share);
   auto key_quad = [&](int g) { return g + (g >> a.pad_shift); };
   const int j0 = jc + tid * q * 4;   // this thread's first token
   int32_t* out = a.idx + (int64_t)row * a.max_k;
   uint16_t* hits = a.hits ? a.hits + (int64_t)row * a.cap : nullptr;
   // the keys are being written: only their address translation is fetched
-  if (search && jc + 4 * tid < hi) prefetch_l2(row_key + max(jc + 4 * tid, 0));
+  if (mine_to_search && jc + 4 * tid < hi) prefetch_l2(row_key + max(jc + 4 * tid, 0));
   pdl_wait();
   pdl_launch_dependents();
 
   // The global reads are issued before the first use of any of them.  A key
   // of 0 means no token (a token's key is at least 1).
   uint4 h0v{0u, 0u, 0u, 0u};
-  if (search && a.hist0 && tid < kBins / 4) h0v = reinterpret_cast<const uint4*>(a.hist0 + (int64_t)row * kBins)[tid];
+  if (mine_to_search && a.hist0 && tid < kBins / 4) h0v = reinterpret_cast<const uint4*>(a.hist0 + (int64_t)row * kBins)[tid];
   // counts of the first digit: taken over, or made from the keys as they come
-  uint32_t* h = CL ? own : sums;
-  if (search) {
-    if (CL && !a.hist0) cluster.barrier_wait();   // A
+  uint32_t* h = multi ? own : sums;
+  if (mine_to_search) {
+    if (multi && !a.hist0) cluster.barrier_wait();   // A
     constexpr int kU = 4;   // quads in flight
     for (int g0 = tid; g0 < nq; g0 += kU * T) {
       float4 f[kU];
@@ -246,6 +258,7 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
       }
     return;
   }
+  if (!mine_to_search) return;
 
   // Add this CTA's non-empty bins to every CTA's sums, and clear them.
   auto push_counts = [&](uint32_t* sum) {
@@ -258,11 +271,11 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
     }
   };
   if (a.hist0) {
-    if (CL) cluster.barrier_wait();   // A
+    if (multi) cluster.barrier_wait();   // A
     if (tid < kBins / 4) reinterpret_cast<uint4*>(sums)[tid] = h0v;
   }
   __syncthreads();
-  if (CL && !a.hist0) {
+  if (multi && !a.hist0) {
     push_counts(sums);
     cluster.sync();
   }
@@ -298,7 +311,7 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
   auto key_of = [&](int i) {   // key i of this thread
     return reinterpret_cast<const uint32_t*>(keys + key_quad(tid * q + (i >> 2)))[i & 3];
   };
-  if (CL || !whole) {
+  if (multi || !whole) {
     // the crossing bin's keys into the list; (keys above) << 16 | (keys in it)
     const uint32_t cnt = (pop(gt) << 16) | pop(in);
     const uint32_t inc = warp_scan(cnt);
@@ -307,30 +320,30 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
     base = __shfl_sync(0xffffffffu, base, 31);
     uint32_t at = (base + inc - cnt) & 0xffffu;
     for (Mask m = in; m; m &= m - 1, ++at)
-      if (at < (uint32_t)a.lcap) list[r * a.lcap + at] = key_of(first(m));
+      if (at < (uint32_t)lcap) list[rs * lcap + at] = key_of(first(m));
     __syncthreads();
   }
-  bool listed = !whole && (my_cnt & 0xffffu) <= (uint32_t)a.lcap;
-  if (CL) {
+  bool listed = !whole && (my_cnt & 0xffffu) <= (uint32_t)lcap;
+  if (multi) {
     const uint32_t nc = my_cnt & 0xffffu;
     if (listed) {
       const int c = tid / kPeerThreads, i0 = tid % kPeerThreads;
       if (c < C && c != r) {
-        const uint32_t* src = list + r * a.lcap;
-        uint32_t* dst = remote(list + r * a.lcap, c);
+        const uint32_t* src = list + r * lcap;
+        uint32_t* dst = remote(list + r * lcap, c);
         for (uint32_t i = i0; i < nc; i += kPeerThreads) dst[i] = src[i];
       }
     }
     if (tid < C) remote(s_cnt, tid)[r] = my_cnt;
     cluster.sync();   // every CTA's list and counts are in place
     listed = !whole;
-    for (int c = 0; c < C; ++c) listed = listed && (s_cnt[c] & 0xffffu) <= (uint32_t)a.lcap;
+    for (int c = 0; c < C; ++c) listed = listed && (s_cnt[c] & 0xffffu) <= (uint32_t)lcap;
   }
-  // f(key, CTA) for every entry of the list: kWarps / C warps take a CTA's part
+  // f(key, CTA) for every entry of the list: kWarps / S warps take a CTA's part
   auto each = [&](auto&& f) {
-    const int per = CL ? kWarps / C : kWarps, c = CL ? warp / per : 0;
-    const uint32_t nc = (CL ? s_cnt[c] : my_cnt) & 0xffffu;
-    for (uint32_t i = (warp - c * per) * 32 + lane; i < nc; i += per * 32) f(list[c * a.lcap + i], c);
+    const int per = kWarps / S, c = warp / per;
+    const uint32_t nc = (multi ? s_cnt[c] : my_cnt) & 0xffffu;
+    for (uint32_t i = (warp - c * per) * 32 + lane; i < nc; i += per * 32) f(list[c * lcap + i], c);
   };
   // the digits that follow, until the crossing bin is taken whole: from counts
   // of the keys that share those found, or, when few listed keys share them,
@@ -367,8 +380,8 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
     if (listed) {
       each([&](uint32_t kv, int) { add(sum, kv); });
     } else {
-      for (Mask m = in; m; m &= m - 1) add(CL ? own : sum, key_of(first(m)));
-      if (CL) {
+      for (Mask m = in; m; m &= m - 1) add(multi ? own : sum, key_of(first(m)));
+      if (multi) {
         __syncthreads();
         push_counts(sum);
         cluster.sync();
@@ -398,7 +411,7 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
   const uint32_t mine = (pop(gt) << 16) | pop(eqm);
   const uint32_t inc = warp_scan(mine);
   if (lane == 31) wcnt[warp] = inc;
-  if (CL && listed) {   // the crossing-bin keys that the CTAs before this one keep
+  if (multi && listed) {   // the crossing-bin keys that the CTAs before this one keep
     uint32_t v = 0;
     each([&](uint32_t kv, int c) {
       if (c < r) v += (kv > top ? 0x10000u : 0u) + (kv == eq ? 1u : 0u);
@@ -410,7 +423,7 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
   const uint32_t wt = lane < kWarps ? wcnt[lane] : 0u;
   const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? wt : 0u) + inc - mine;
   uint32_t pos = before >> 16, eq_rank = before & 0xffffu;
-  if (CL) {
+  if (multi) {
     if (listed || whole0) {
       pos += s_before >> 16;   // (0 when the first digit decided)
       eq_rank += s_before & 0xffffu;
@@ -472,21 +485,24 @@ int select_hist_bins() { return kBins; }
 
 cudaError_t launch_select(const SelectArgs& a0, int sms, cudaStream_t st) {
   SelectArgs a = a0;
-  // CTAs per row: more until a CTA has at most kChunk keys, while twice as
-  // many still fit `sms`; else as few as hold kChunkMax each.  Measured (us a
-  // selection after the scoring, one against four or eight CTAs): 32K x 4
-  // rows 9.8 / 7.4, 64K x 8 13.4 / 11.1, 16K x 4 8.0 / 7.6, per-KV-head 16K x
-  // 16 rows -1.5 with 2 -> 4; 4K rows are faster in one CTA (5.5 against 7.1).
+  // CTAs per row: one up to kAlone keys; then more until a CTA has at most
+  // kChunk keys, while twice as many still fit `sms`; else as few as hold
+  // kChunkMax each.  Measured (us a selection after the scoring, one against four
+  // or eight CTAs): 32K x 4 rows 9.8 / 7.4, 64K x 8 13.4 / 11.1, 16K x 4 8.0 / 7.6,
+  // per-KV-head 16K x 16 rows -1.5 with 2 -> 4; alone, 16 rows of 8K 6.7 in one
+  // CTA and 7.6 in two or four.
   const int rows = a.B * a.rows_per_seq;
   int C = 1;
-  while (C < kMaxCluster && (a.cap + C - 1) / C > (2 * C * rows <= sms ? kChunk : kChunkMax)) C <<= 1;
-  const int share = (((a.cap + 3 + C - 1) / C) + 3) & ~3;   // of a CTA, at most (see the kernel)
+  while (a.cap > kAlone && C < kMaxCluster && (a.cap + C - 1) / C > (2 * C * rows <= sms ? kChunk : kChunkMax)) C <<= 1;
+  int share = (((a.cap + 3 + C - 1) / C) + 3) & ~3;   // of a CTA, at most (see the kernel)
+  if (C > 1) share = std::max(share, kAlone);
   const int nq = share / 4, counts = (C > 1 ? 4 : 3) * kBins;
   // the spare quads, where they fit beside a list of full size
   a.pad_shift = (nq + nq / 8 + 1) * 4 + counts + kListMax <= kSelSmem / 4 ? 3 : 31;
   const int key_words = (nq + (nq >> a.pad_shift) + 1) * 4;
   a.lcap = std::min(kListMax, kSelSmem / 4 - counts - key_words) / C;
   a.list_words = (a.lcap * C + 3) & ~3;
+  a.alone_max = kAlone;
   const size_t smem = (size_t)(counts + a.list_words + key_words) * 4;
   const bool m32 = nq <= 8 * T;   // at most 32 keys per thread
   if (C > 1) return m32 ? launch_select_t<true, uint32_t>(a, C, smem, st) : launch_select_t<true, uint64_t>(a, C, smem, st);

@@ -76,3 +76,51 @@ def test_select_longest_row(H, oracle_mod):
     desc = H.make_desc(q, K.expand(1, 1, cap + 1, 128))
     with pytest.raises(H.HillError):
         H.hill_topk_select(desc, torch.zeros(1, cap + 1, device="cuda"), one(cap), one(1), 1, idx, count)
+
+
+@pytest.mark.parametrize("kind", ["random", "narrow", "ties", "flat", "bins"])
+@pytest.mark.parametrize("cap", [8193, 16385, 40002, 131135])
+def test_short_rows_of_a_large_cache(H, oracle_mod, cap, kind):
+    """Rows at and around the 8192 ranked tokens up to which a cluster's first CTA works alone, for every place of a
+    row's first key in its 16 bytes (odd capacities), beside rows that all CTAs search; budgets at both ends."""
+    lens = [1, 2, 33, 4096, 8188, 8189, 8190, 8191, 8192, 8193, 8000, cap]
+    budgets = [1, 1, 32, 64, 8187, 1, 819, 65, 4096, 700, 8000, 1000]
+    rows = len(lens)
+    x = _keys(kind, rows, cap, cap)
+    K = torch.zeros(rows, 1, 1, 128, dtype=torch.float16, device="cuda").expand(rows, 1, cap, 128)
+    desc = H.make_desc(torch.zeros(rows, 1, 128, dtype=torch.float16, device="cuda"), K)
+    dev = lambda v: torch.tensor(v, dtype=torch.int32, device="cuda")  # noqa: E731
+    for recent, hits in ((0, None), (3, torch.randint(0, 65536, (rows, cap), generator=torch.Generator().manual_seed(5)))):
+        max_k = max(budgets) + recent
+        idx = torch.full((rows, max_k), -9, dtype=torch.int32, device="cuda")
+        count = torch.full((rows,), -9, dtype=torch.int32, device="cuda")
+        h0 = None if hits is None else hits.numpy().astype(np.uint16)
+        hd = None if h0 is None else torch.from_numpy(h0.view(np.int16).copy()).cuda()
+        H.hill_topk_select_bkp(desc, x.cuda(), dev(lens), dev(budgets), recent, max_k, idx, count, hd)
+        H.hill_sync_status()
+        want_i, want_c, rc, want_h = oracle_mod.bkp_select(x.numpy(), lens, budgets, recent, max_k, h0)
+        assert np.array_equal(count.cpu().numpy(), want_c) and np.array_equal(idx.cpu().numpy(), want_i)
+        if h0 is not None:
+            assert np.array_equal(hd.cpu().numpy().view(np.uint16), want_h)
+
+
+@pytest.mark.parametrize("cap", [16385, 70001])
+def test_short_rows_counted_by_the_normalisation(H, cap):
+    """The same with the leading digits counted by the ATTN normalisation."""
+    lens, g = [1000, 8191, 8192, 8193, 1, cap], torch.Generator(device="cuda").manual_seed(cap)
+    K = torch.randn(len(lens), 2, cap, 128, generator=g, device="cuda").half()
+    q = torch.randn(len(lens), 4, 128, generator=g, device="cuda").half()
+    kept = [max(1, m // 7) for m in lens]
+    dev = lambda v: torch.tensor(v, dtype=torch.int32, device="cuda")  # noqa: E731
+    scores = torch.zeros(len(lens), cap, device="cuda")
+    idx = torch.zeros(len(lens), max(kept), dtype=torch.int32, device="cuda")
+    count = torch.zeros(len(lens), dtype=torch.int32, device="cuda")
+    desc = H.make_desc(q, K)
+    H.hill_evict_step(desc, q, K, None, dev(lens), dev(kept), max(kept), 0, None, scores, idx, count, None,
+                      H.alloc_workspace(desc, 0, max(kept)))
+    H.hill_sync_status()
+    assert count.tolist() == kept
+    for b, m in enumerate(lens):
+        order = torch.sort(scores[b, :m], descending=True, stable=True).indices[:kept[b]]
+        assert torch.equal(idx[b, :kept[b]].long(), order.sort().values)
+        assert torch.all(idx[b, kept[b]:] == -1)
