@@ -2,10 +2,12 @@
 // workspace layout and the launch sequence of each call.
 #include <cudaTypedefs.h>
 
+#include <unistd.h>
+
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <mutex>
-#include <random>
 
 #include "../../include/hill.h"
 #include "hill_internal.h"
@@ -36,13 +38,16 @@ cudaError_t counted(cudaError_t e, int kernels) {
   return e;
 }
 
-// The tag of a scoring launch whose tail is claimed: 63 random bits, odd (a
-// counter of the process from a random start, mixed; splitmix64, Steele et al.
-// 2014).
+// The tag of a scoring launch whose tail is claimed: odd, a counter of the
+// process from a random start, mixed (splitmix64, Steele et al. 2014).  The
+// start comes from the system without a call that may throw; where the system
+// has none to give, from the clock.
 unsigned long long next_claim_tag() {
   static const uint64_t start = [] {
-    std::random_device rd;
-    return ((uint64_t)rd() << 32) ^ rd();
+    uint64_t v = 0;
+    if (getentropy(&v, sizeof v) != 0)
+      v = (uint64_t)std::chrono::steady_clock::now().time_since_epoch().count() * 0x9e3779b97f4a7c15ull;
+    return v;
   }();
   static std::atomic<uint64_t> n{0};
   uint64_t z = start + (n.fetch_add(1, std::memory_order_relaxed) + 1) * 0x9e3779b97f4a7c15ull;

@@ -143,3 +143,11 @@ def test_product_never_imports_the_oracle():
                 text = open(os.path.join(dirpath, f)).read()
                 assert not re.search(r"^\s*(import|from)\s+oracle\b", text, flags=re.M), f
                 assert "hill_oracle" not in text and "liboracle" not in text, f
+
+
+def test_no_throwing_source_of_random_bits(lib):
+    """The claim tags' random start must not come from std::random_device, which throws where the system has no source
+    of random bits: the exception would cross the C entry and end the process."""
+    from paper_2602_18750_gb300 import hill
+    out = subprocess.run(["nm", "-D", "--undefined-only", hill.LIB_PATH], capture_output=True, text=True, check=True)
+    assert "random_device" not in out.stdout
