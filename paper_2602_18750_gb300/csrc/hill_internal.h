@@ -67,7 +67,7 @@ struct FinalizeArgs {
   int recent;         // tokens j >= len - min(recent, len) are left out of hist0 (pinned, not ranked)
   int kvh;            // 1: scores/accum are [B][Hkv][cap], the sum over each KV head's G query heads
   int Hkv;
-  float2* stats;      // [B][H] (max, 1/sum) per head, written by hill_attn_stats_kernel in the split step
+  float2* stats;      // [B][H] (max, 1/sum) per head, written by hill_attn_stats_kernel where the normalisation takes two kernels
   int tpt;            // blocks of tokens per finalize CTA (set by the launcher)
 };
 

@@ -6,7 +6,9 @@
 // range of items [x * per, (x + 1) * per), so it meets one or two sequences
 // and loads their queries and flushes their partials once (measured faster
 // than dealing items round robin, by 4 % at 32K and more for short
-// sequences, where round robin changes sequence at every item).  The KV
+// sequences, where round robin changes sequence at every item).  Of a long
+// 16-bit ATTN stream only the first 13/16 are dealt out so; the rest is
+// claimed tile by tile by warps that are free (struct Units).  The KV
 // heads g of an item are dealt to the warps (g mod kNW).  Every warp streams
 // its own (item, g)
 // sequence through a private ring of kSW shared-memory stages: lane 0 issues
@@ -24,11 +26,12 @@
 //   ATTN: every logit, pre-scaled by log2 e, is written to a [B][H][cap]
 //         buffer; each lane keeps a running (max, sum 2^(z2 - max)) of its
 //         own tokens per head in registers, and the lanes of a head are
-//         combined once, when the CTA leaves a sequence, into one partial per
-//         (sequence, head, CTA).  hill_attn_finalize_kernel combines the
-//         partials and forms s[b,j] = sum_h exp(z[b,h,j] - m_bh) / L_bh; with
-//         more than one such CTA per SM hill_attn_stats_kernel first combines
-//         the partials once per (sequence, head).
+//         combined once, when the CTA leaves a sequence or a claimed tile,
+//         into one partial per (sequence, head, unit of work).
+//         hill_attn_finalize_kernel combines the partials and forms s[b,j] =
+//         sum_h exp(z[b,h,j] - m_bh) / L_bh; with many such CTAs or partials
+//         hill_attn_stats_kernel first combines the partials once per
+//         (sequence, head) (launch_attn_finalize).
 //
 // The query rows of a warp's heads are held as mma B fragments in registers
 // for the whole sequence.  Before its dependency wait the kernel builds its
@@ -119,10 +122,10 @@ struct Units {
 // The claim counters lie in the caller's workspace, whose contents are
 // arbitrary before a call, and no kernel of the call runs before this one.  So
 // the first warp that needs a counter opens it: a counter counts only under
-// the tag of its launch (odd, 64 random bits drawn by the host), which is put
-// in place in two steps (tag - 1 while the count is being zeroed).  The
-// normalisation, which runs when every claim is over, takes the tags away
-// again, so that a graph's next replay finds them closed.  A warp waits here
+// the tag of its launch (odd; the host draws 63 bits), which is put in place in
+// two steps (tag - 1 while the count is being zeroed).  The normalisation, which
+// runs when every claim is over, takes the tags away again whatever the
+// lengths, so that a graph's next replay finds them closed.  A warp waits here
 // only for another one that is between two stores; the wait is bounded.
 __device__ __noinline__ void open_claims(ClaimCounter* c, unsigned long long tag, unsigned* err) {
   volatile unsigned long long* t = &c->tag;

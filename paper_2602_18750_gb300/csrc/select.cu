@@ -168,7 +168,7 @@ __global__ void __launch_bounds__(T) hill_select_kernel(const SelectArgs a) {
   const int s0 = (int)((reinterpret_cast<uintptr_t>(row_key) >> 2) & 3u);
   // A short row of a large cache is searched by the cluster's first CTA alone,
   // without the exchanges.  4 rows in a cache of 16K, four CTAs each / alone
-  // (us): 1000 tokens 6.4 / 4.6, 4000 7.5 / 5.2, 6000 6.7 / 5.7, 8000 6.9 / 6.0.
+  // (us): 1000 tokens 6.4 / 4.6, 6000 6.7 / 5.7, 8000 6.9 / 6.0.
   const bool alone = CL && older + s0 <= a.alone_max;
   const bool multi = CL && !alone;   // the CTAs search together
   const int S = alone ? 1 : C, rs = alone ? 0 : r;   // the CTAs that search; this one among them

@@ -69,7 +69,7 @@ def test_attention_over_every_split(H, case, dtype):
         H.hill_sync_status()
         check_attn(out.cpu().numpy(), ref)
         if first is not None:
-            assert torch.equal(out, first), "the merge order must not depend on which CTA arrives last"
+            assert torch.equal(out, first), "the order of the merge is fixed"
         first = out.clone()
         out.fill_(float("nan"))
 

@@ -215,6 +215,13 @@ def test_claimed_tail_of_a_large_cache(Hq, Hkv, dtype, lens, claimed):
     H.hill_evict_step(desc, q, K, None, lens_t, kept, 50, 0, accum, scores, idx, torch.empty_like(kept), None, ws)
     H.hill_sync_status()
     assert torch.equal(scores, first) and torch.equal(accum, first)
+    # and with sets of their own for the KV heads, whose importance adds up to the sequence's
+    group = torch.zeros(B, Hkv, cap, device="cuda")
+    H.hill_evict_step_kvh(desc, q, K, None, lens_t, kept, 50, 0, None, group,
+                          torch.zeros(B, Hkv, 50, dtype=torch.int32, device="cuda"),
+                          torch.zeros(B, Hkv, dtype=torch.int32, device="cuda"), None, ws)
+    H.hill_sync_status()
+    assert torch.all((group.double().sum(1) - first.double()).abs() <= 1e-5 * first.double())
     for b, m in enumerate(lens):
         assert not scores[b, m:].any()
         if m == 0:
