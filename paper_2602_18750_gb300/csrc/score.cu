@@ -108,13 +108,13 @@ __device__ __forceinline__ int find_seq(const int* tstart, int B, int item) {
 // hill_score on 8 x 1000 tokens in a cache for 8 x 8K takes 14.1 us with the even
 // split and 23.2 with claims, on 16 x 200 in one for 16 x 4K 10.1 and 18.1.
 struct Units {
-  int per, dyn0, grid;   // items of a share; the first item claimed (n_items: none)
+  int per, dyn0, grid;   // items of a share; the first item claimed (INT_MAX: none, folded away in kernels without claims)
   __device__ __forceinline__ Units(int n_items, int grid_, int claim_min) {
     grid = grid_;
     const int share = n_items / 16 * kShare16 / grid;
     const bool claims = claim_min > 0 && n_items >= claim_min && share >= kMinShare;
     per = claims ? share : (n_items + grid - 1) / grid;
-    dyn0 = claims ? grid * per : n_items;
+    dyn0 = claims ? grid * per : 0x7fffffff;
   }
   __device__ __forceinline__ int of(int item) const { return item < dyn0 ? item / per : grid + (item - dyn0); }
 };
