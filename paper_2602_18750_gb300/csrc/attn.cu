@@ -739,16 +739,21 @@ cudaError_t launch_attn_cl(const AttnArgs& a, int sms, cudaStream_t st, bool* do
   const int64_t passes = (a.Gs + 15) / 16;
   if (C == 0 || even > 32 || rounds > even + even / 4 + 3 * passes) return cudaSuccess;
   // The counts are not known here.  With one sequence at max_k and the others
-  // nearly empty the even split has only that one's batches to deal out
-  // (`one` rounds), while its clusters still take all their rounds, at about 1
-  // us each.  Measured, even split / clusters, equal counts and one long one (us,
-  // rounds - one in brackets): 32 heads, 8 x 819 18.8 / 14.9, [819, 7 x 50] 10.3 /
-  // 10.2 (6); 8 KV heads, 16 x 1638 23.4 / 15.9, 11.0 / 11.4 (6); 4 x 6553 19.7 /
-  // 16.0, 12.0 / 11.9 (5); but 32 heads, 4 x 2457 31.8 / 28.4 and [3277, 3 x 200]
-  // 13.8 / 17.6 (10); 40 heads, 6 x 1500 35.5 / 31.4, [1500, 5 x 50] 10.4 / 15.5 (10)
+  // nearly empty the even split has only that one's batches to deal out (`one`
+  // rounds), while its clusters still take all their rounds, at 0.5 to 1 us each.
+  // Measured, even split / clusters (us) with equal counts, counts of 50-100 %,
+  // half of them at 1/8, and one beside 50s; rounds - one in brackets:
+  //   32 heads, 8 x 819 (6)  18.9 / 14.7  15.7 / 12.7  13.7 / 10.6  10.3 / 10.2
+  //             8 x 947 (7)  24.8 / 20.6  16.0 / 14.4  13.7 / 11.9  10.3 / 11.3
+  //             4 x 2300 (7) 30.8 / 26.9  22.0 / 20.1  15.6 / 14.4  12.4 / 13.1
+  //             8 x 1100 (8) 29.6 / 25.2  18.8 / 16.9  15.4 / 13.5  10.3 / 12.4
+  //             4 x 2600 (8) 34.0 / 30.9  26.9 / 25.5  16.0 / 17.0  12.5 / 15.2
+  //             4 x 3277 (10) 40.1 / 37.1  33.2 / 31.4  23.9 / 21.8  12.6 / 17.4
+  // (beside empty ones up to 2.6 us lost at 7).  The line lies where the last
+  // column loses less than the others gain.
   const int units = a.kvh ? a.B * a.Hkv : a.B;
   const int64_t one = (triples / units * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
-  if (units > 1 && rounds > one + 6 * passes) return cudaSuccess;
+  if (units > 1 && rounds > one + 1 + 6 * passes) return cudaSuccess;
   *done = true;
   const dim3 grid((unsigned)(triples * C));
   return half ? launch_pdl(hill_sparse_attn_kernel<DT, G, true, kAW / 2>, grid, dim3(kAThreads / 2), AttnCfg::smem(kAW / 2),

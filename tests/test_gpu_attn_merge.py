@@ -76,6 +76,7 @@ def test_attention_over_every_split(H, case, dtype):
 
 @pytest.mark.parametrize("B,Hq,Hkv,n,kept,max_k,launches", [
     (8, 32, 32, 4096, [819] * 8, 819, 1), (8, 32, 32, 4096, [819] + [0] * 7, 819, 1),
+    (8, 32, 32, 4096, [947, 0, 1, 31, 600, 0, 0, 33], 947, 1),
     (4, 32, 32, 4096, [3277, 200, 0, 200], 3277, 2),    # one long sequence: its batches over all warps
     (6, 40, 40, 2048, [1500, 50, 50, 0, 50, 1], 1500, 2),
     (1, 32, 32, 4096, [3277], 3277, 1), (2, 32, 32, 4096, [3277, 1], 3277, 1),
