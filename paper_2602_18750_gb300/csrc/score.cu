@@ -709,7 +709,7 @@ __global__ void __maxnreg__(kScoreMaxRegs) hill_score_kernel(const __grid_consta
 // head.
 constexpr int kFinThreads = 256;                   // threads (= tokens) of a CTA
 constexpr int kFinHB = 4;                          // heads of a warp whose partials are combined together
-constexpr int kFinU = 5;                           // partials per lane and head held in registers
+constexpr int kFinU = 5;                           // partials per lane and head held in registers at a time
 constexpr int kHistBins = 2048;                    // leading 11 bits of the order-preserving key
 constexpr int kFinZ = 32;                          // logits per token held in registers
 constexpr int kFinMaxTpt = 16;                     // token blocks per CTA at most (split step)
@@ -717,39 +717,36 @@ constexpr int kFinMaxTpt = 16;                     // token blocks per CTA at mo
 __device__ __forceinline__ int pad8(int h) { return (h + 7) & ~7; }
 
 // The (max, 1/sum) of every head of sequence b from its ns per-CTA partials:
-// a warp takes kFinHB of its heads at a time.
+// a warp takes kFinHB of its heads at a time, kFinU partials per lane and head in
+// flight (one KV head has up to 8 partials per scoring CTA: hill_score on 4096
+// tokens of 32 query heads 11.8 us; with one partial per lane at a time past the
+// first kFinU 39.8).
 __device__ __forceinline__ void combine_partials(const FinalizeArgs& a, int b, int ns, float2* wt) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   constexpr int NW = kFinThreads / 32, HB = kFinHB;
   const float2* pb = a.partials + (int64_t)b * a.H * a.nslot;
   for (int h0 = warp; h0 < a.H; h0 += NW * HB) {
-    float2 p[HB][kFinU];
-#pragma unroll
-    for (int i = 0; i < HB; ++i)
-#pragma unroll
-      for (int u = 0; u < kFinU; ++u) {
-        const int h = h0 + NW * i, s = lane + 32 * u;
-        p[i][u] = h < a.H && s < ns ? pb[(int64_t)h * a.nslot + s] : make_float2(-INFINITY, 0.f);
-      }
     float m[HB], l[HB];
 #pragma unroll
-    for (int i = 0; i < HB; ++i) {
-      m[i] = -INFINITY;
+    for (int i = 0; i < HB; ++i) m[i] = -INFINITY, l[i] = 0.f;
+    // 32 * kFinU slots of each head at a time, all loads in flight
+    for (int s0 = 0; s0 < ns; s0 += 32 * kFinU) {
+      float2 p[HB][kFinU];
 #pragma unroll
-      for (int u = 0; u < kFinU; ++u) m[i] = fmaxf(m[i], p[i][u].x);
-      l[i] = 0.f;
+      for (int i = 0; i < HB; ++i)
 #pragma unroll
-      for (int u = 0; u < kFinU; ++u) l[i] += p[i][u].y > 0.f ? p[i][u].y * ex2(p[i][u].x - m[i]) : 0.f;
-    }
-    // slots past 32 * kFinU (the dealing kernel's): a running maximum
-    for (int s0 = 32 * kFinU; s0 < ns; s0 += 32) {
+        for (int u = 0; u < kFinU; ++u) {
+          const int h = h0 + NW * i, s = s0 + lane + 32 * u;
+          p[i][u] = h < a.H && s < ns ? pb[(int64_t)h * a.nslot + s] : make_float2(-INFINITY, 0.f);
+        }
 #pragma unroll
       for (int i = 0; i < HB; ++i) {
-        const int h = h0 + NW * i, s = s0 + lane;
-        const float2 q = h < a.H && s < ns ? pb[(int64_t)h * a.nslot + s] : make_float2(-INFINITY, 0.f);
-        if (!(q.y > 0.f)) continue;
-        const float mn = fmaxf(m[i], q.x);
-        l[i] = (l[i] > 0.f ? l[i] * ex2(m[i] - mn) : 0.f) + q.y * ex2(q.x - mn);
+        float mn = m[i];
+#pragma unroll
+        for (int u = 0; u < kFinU; ++u) mn = fmaxf(mn, p[i][u].x);
+        l[i] = l[i] > 0.f ? l[i] * ex2(m[i] - mn) : 0.f;
+#pragma unroll
+        for (int u = 0; u < kFinU; ++u) l[i] += p[i][u].y > 0.f ? p[i][u].y * ex2(p[i][u].x - mn) : 0.f;
         m[i] = mn;
       }
     }
@@ -1122,15 +1119,15 @@ cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t s
       a.tpt <<= 1;
   // The partials are combined once per (b, h) in a kernel of their own instead
   // of once per CTA with more than two CTAs per SM (attn_finalize_waves), and
-  // with more than one where a head has more partials than a warp holds in
-  // registers.  Measured, hill_score, one / two kernels (us): 4 x 10K tokens, 8
-  // KV heads (38 partials a head) 18.5 / 19.8, with 1000 tokens in each 6.9 / 6.9
-  // and issued eagerly 11.0 / 12.7; 8 x 6000, 32 KV heads 60.1 / 60.0, with 600 in
-  // each 9.8 / 10.3; 1 x 64K, 8 KV heads (152 partials) 25.6 / 26.0; 16 x 4K of
-  // one KV head (76) 16.6 / 18.0, but 4 x 16K of one (304), scores to selection,
-  // 27.7 / 23.8.
+  // with more than one where a head has more partials than a warp loads in two
+  // rounds.  Measured, hill_score, one / two kernels (us): 4 x 10K tokens, 8 KV
+  // heads (38 partials a head) 18.5 / 19.8, with 1000 tokens in each 6.9 / 6.9 and
+  // issued eagerly 11.0 / 12.7; 8 x 6000, 32 KV heads 60.1 / 60.0, with 600 in each
+  // 9.8 / 10.3; 1 x 64K, 8 KV heads (152 partials) 25.6 / 26.0; one KV head, 16 x
+  // 4K (76) 16.6 / 18.0, 4 x 16K (304) 16.9 / 17.5, 2 x 32K (608) 17.8 / 16.8, 1 x
+  // 64K (1216) 18.9 / 15.7.
   if (two_kernel || attn_finalize_waves(a.B, a.cap, sms) > 2 ||
-      (attn_finalize_waves(a.B, a.cap, sms) > 1 && a.score_grid * a.spc / a.B > 32 * kFinU)) {
+      (attn_finalize_waves(a.B, a.cap, sms) > 1 && a.score_grid * a.spc / a.B > 2 * 32 * kFinU)) {
     *kernels = 2;
     const int W = a.claim_min > 0 ? 4 : 1;   // warps per (b, h)
     const dim3 sgrid((a.B * a.H * W + kStatsWarps - 1) / kStatsWarps);

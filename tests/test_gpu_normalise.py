@@ -14,6 +14,8 @@ CASES = [
     (2, 9, 3, [257, 0]),
     (1, 32, 1, [6000]),              # 1216 partials per head, combined in the one kernel
     (3, 8, 1, [30000, 16000, 1]),    # the same in two kernels
+    (1, 71, 1, [8000]),              # and over three passes of heads
+    (2, 20, 2, [5000, 40]),
     (2, 28, 4, [3001, 2999]),
     (2, 64, 8, [9000, 4097]),        # two rounds of 32 heads
     (1, 72, 8, [70001]),             # three, in two kernels
@@ -97,7 +99,8 @@ def _claims(ws, desc):
 
 @pytest.mark.parametrize("B,Hq,Hkv,n,launches", [
     (4, 32, 8, 10000, 2), (1, 32, 8, 65536, 2), (16, 32, 1, 4096, 2), (8, 32, 32, 8192, 2),   # up to two blocks per SM
-    (4, 32, 1, 16384, 3),                       # with more partials per head than a warp's registers hold
+    (4, 32, 1, 16384, 2), (1, 32, 1, 4096, 2),   # several rounds of partials per head
+    (1, 32, 1, 65536, 3), (2, 32, 1, 32000, 3),  # more than two blocks per SM or two rounds of partials
     (1, 32, 8, 80000, 3), (1, 32, 32, 80000, 3),
 ])
 def test_launches_of_the_normalisation(B, Hq, Hkv, n, launches):
