@@ -103,10 +103,11 @@ __device__ __forceinline__ int find_seq(const int* tstart, int B, int item) {
 // 178.8 -> 167.9 us, on 8 x 64K 887.9 -> 860.0 (11/16 and 12/16 the same within
 // 1 %, 14/16 2 % slower).  Opening the counters and a flush of the statistics
 // per claim cost 3-5 us, so short streams keep the even split: claim_min is the
-// number of tiles from which the rest is claimed (0: never; run_score).  The
-// tiles counted are those of the lengths at hand, not of the cache's capacity:
-// hill_score on 8 x 1000 tokens in a cache for 8 x 8K takes 14.1 us with the even
-// split and 23.2 with claims, on 16 x 200 in one for 16 x 4K 10.1 and 18.1.
+// number of tiles from which the rest is claimed (0: never; claim_min_for in
+// api.cu).  The tiles counted are those of the lengths at hand, not of the
+// cache's capacity: hill_score on 8 x 1638 tokens in a cache for 8 x 32K takes
+// 21.0 us with the even split and 26.1 with claims, on 4096 in one for 128K 9.3
+// and 17.0.
 struct Units {
   int per, dyn0, grid;   // items of a share; the first item claimed (INT_MAX: none, folded away in kernels without claims)
   __device__ __forceinline__ Units(int n_items, int grid_, int claim_min) {
