@@ -952,10 +952,12 @@ __global__ void __launch_bounds__(kFinThreads, STATS ? 4 : 2) hill_attn_finalize
 
 // Combine the per-unit (max, sum) partials of one (b, h) into its softmax
 // statistics (max, 1 / sum) in the base-2 scale: W warps per pair, each lane
-// taking every 32 W-th partial with a running maximum, the lanes then merged
-// by shuffles and the warps in shared memory.  Used ahead of
-// hill_attn_finalize_kernel<true, *> when the normalisation has many CTAs per
-// sequence; W > 1 when tiles were claimed, which leaves a partial per tile.
+// taking every 32 W-th partial, kStatsPer at a time under their common maximum
+// (a running one per partial scales the sum more often: scores of 4 x 16K tokens
+// on one KV head were 2.68e-7 from 64 bits by it, 2.60e-7 now), the lanes then
+// merged by shuffles and the warps in shared memory.  Used ahead of
+// hill_attn_finalize_kernel<true, *> where launch_attn_finalize says; W > 1 when
+// tiles were claimed, which leaves a partial per tile.
 constexpr int kStatsWarps = 8;
 constexpr int kStatsPer = 8;   // partials per lane whose loads are in flight together
 
@@ -996,13 +998,13 @@ __global__ void __launch_bounds__(kStatsWarps * 32) hill_attn_stats_kernel(Final
       const int s = s0 + 32 * W * u;
       p[u] = s < ns ? pb[s] : make_float2(-INFINITY, 0.f);
     }
+    float mn = m;   // (their maximum first, so that every term is scaled once)
 #pragma unroll
-    for (int u = 0; u < kStatsPer; ++u) {
-      if (!(p[u].y > 0.f)) continue;
-      const float mn = fmaxf(m, p[u].x);
-      l = l * ex2(m - mn) + p[u].y * ex2(p[u].x - mn);
-      m = mn;
-    }
+    for (int u = 0; u < kStatsPer; ++u) mn = fmaxf(mn, p[u].x);
+    l = l > 0.f ? l * ex2(m - mn) : 0.f;
+#pragma unroll
+    for (int u = 0; u < kStatsPer; ++u) l += p[u].y > 0.f ? p[u].y * ex2(p[u].x - mn) : 0.f;
+    m = mn;
   }
   auto merge = [&](float mo, float lo) {
     const float mn = fmaxf(m, mo);
@@ -1120,15 +1122,15 @@ cudaError_t launch_attn_finalize(const FinalizeArgs& a0, int sms, cudaStream_t s
       a.tpt <<= 1;
   // The partials are combined once per (b, h) in a kernel of their own instead
   // of once per CTA with more than two CTAs per SM (attn_finalize_waves), and
-  // with more than one where a head has more partials than a warp loads in two
-  // rounds.  Measured, hill_score, one / two kernels (us): 4 x 10K tokens, 8 KV
+  // with more than one where a head has more partials than a warp loads in one
+  // round.  Measured, hill_score, one / two kernels (us): 4 x 10K tokens, 8 KV
   // heads (38 partials a head) 18.5 / 19.8, with 1000 tokens in each 6.9 / 6.9 and
   // issued eagerly 11.0 / 12.7; 8 x 6000, 32 KV heads 60.1 / 60.0, with 600 in each
   // 9.8 / 10.3; 1 x 64K, 8 KV heads (152 partials) 25.6 / 26.0; one KV head, 16 x
-  // 4K (76) 16.6 / 18.0, 4 x 16K (304) 16.9 / 17.5, 2 x 32K (608) 17.8 / 16.8, 1 x
-  // 64K (1216) 18.9 / 15.7.
+  // 4K (76) 16.6 / 18.0, 4 x 16K (304) 16.9 / 17.5, the step on 4 of 8-16K 33.0 /
+  // 32.6, 2 x 32K (608) 17.8 / 16.8, 1 x 64K (1216) 18.9 / 15.7.
   if (two_kernel || attn_finalize_waves(a.B, a.cap, sms) > 2 ||
-      (attn_finalize_waves(a.B, a.cap, sms) > 1 && a.score_grid * a.spc / a.B > 2 * 32 * kFinU)) {
+      (attn_finalize_waves(a.B, a.cap, sms) > 1 && a.score_grid * a.spc / a.B > 32 * kFinU)) {
     *kernels = 2;
     const int W = a.claim_min > 0 ? 4 : 1;   // warps per (b, h)
     const dim3 sgrid((a.B * a.H * W + kStatsWarps - 1) / kStatsWarps);

@@ -99,8 +99,8 @@ def _claims(ws, desc):
 
 @pytest.mark.parametrize("B,Hq,Hkv,n,launches", [
     (4, 32, 8, 10000, 2), (1, 32, 8, 65536, 2), (16, 32, 1, 4096, 2), (8, 32, 32, 8192, 2),   # up to two blocks per SM
-    (4, 32, 1, 16384, 2), (1, 32, 1, 4096, 2),   # several rounds of partials per head
-    (1, 32, 1, 65536, 3), (2, 32, 1, 32000, 3),  # more than two blocks per SM or two rounds of partials
+    (1, 32, 1, 4096, 2), (2, 32, 1, 16000, 2),   # several rounds of partials per head
+    (4, 32, 1, 16384, 3), (1, 32, 1, 65536, 3),  # the same on more than one block per SM
     (1, 32, 8, 80000, 3), (1, 32, 32, 80000, 3),
 ])
 def test_launches_of_the_normalisation(B, Hq, Hkv, n, launches):
