@@ -722,9 +722,11 @@ cudaError_t launch_attn_cl(const AttnArgs& a, int sms, cudaStream_t st, bool* do
   cudaError_t e = triples <= sms ? attn_cluster_size<DT, G, kAW>(triples, nb, sms, &c8, &r8) : cudaSuccess;
   if (e == cudaSuccess) e = attn_cluster_size<DT, G, kAW / 2>(triples, nb, sms, &c4, &r4);
   if (e != cudaSuccess) return e;
-  // CTAs of 4 warps, which spread a (b, g) over twice as many SMs, unless they
-  // take more rounds
-  const bool half = c8 == 0 || (c4 > 0 && r4 <= r8);
+  // with several sequences CTAs of 4 warps, which spread a (b, g) over twice as
+  // many SMs, unless they take more rounds (one sequence: its pairs are alike, and
+  // beside a K stream fewer, larger CTAs wait less: 1 x 64K, k 50 %, pipelined step
+  // 146 us per layer against 151)
+  const bool half = c8 == 0 || (c4 > 0 && (a.B > 1 ? r4 <= r8 : r4 < r8));
   const int C = half ? c4 : c8, rounds = half ? r4 : r8;
   const int64_t even = (triples * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
   // A round (one more batch per warp) costs about 1.6 us where latency bounds
@@ -751,9 +753,8 @@ cudaError_t launch_attn_cl(const AttnArgs& a, int sms, cudaStream_t st, bool* do
   //             4 x 3277 (10) 40.1 / 37.1  33.2 / 31.4  23.9 / 21.8  12.6 / 17.4
   // (beside empty ones up to 2.6 us lost at 7).  The line lies where the last
   // column loses less than the others gain.
-  const int units = a.kvh ? a.B * a.Hkv : a.B;
-  const int64_t one = (triples / units * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
-  if (units > 1 && rounds > one + 1 + 6 * passes) return cudaSuccess;
+  const int64_t one = (triples / a.B * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
+  if (a.B > 1 && rounds > one + 1 + 6 * passes) return cudaSuccess;
   *done = true;
   const dim3 grid((unsigned)(triples * C));
   return half ? launch_pdl(hill_sparse_attn_kernel<DT, G, true, kAW / 2>, grid, dim3(kAThreads / 2), AttnCfg::smem(kAW / 2),
