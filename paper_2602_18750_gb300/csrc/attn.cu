@@ -751,10 +751,14 @@ cudaError_t launch_attn_cl(const AttnArgs& a, int sms, cudaStream_t st, bool* do
   //             8 x 1100 (8) 29.6 / 25.2  18.8 / 16.9  15.4 / 13.5  10.3 / 12.4
   //             4 x 2600 (8) 34.0 / 30.9  26.9 / 25.5  16.0 / 17.0  12.5 / 15.2
   //             4 x 3277 (10) 40.1 / 37.1  33.2 / 31.4  23.9 / 21.8  12.6 / 17.4
-  // (beside empty ones up to 2.6 us lost at 7).  The line lies where the last
-  // column loses less than the others gain.
+  //   4 heads per KV head, 8 KV heads,
+  //             16 x 2200 (8) 34.5 / 26.8  25.0 / 18.9  19.7 / 15.0  11.2 / 13.6
+  //             8 x 4600 (8) 32.3 / 27.6  22.1 / 19.5  17.0 / 15.2  11.7 / 13.8
+  //             8 x 5600 (10) 37.4 / 32.7  29.1 / 26.3  19.6 / 18.3  12.0 / 15.9
+  // (beside empty ones up to 2.7 us lost within the lines).  The lines, 7 and
+  // for groups 8, lie where the last column loses less than the others gain.
   const int64_t one = (triples / a.B * nb + (int64_t)sms * kAW - 1) / ((int64_t)sms * kAW);
-  if (a.B > 1 && rounds > one + 1 + 6 * passes) return cudaSuccess;
+  if (a.B > 1 && rounds > one + (a.Gs > 1 ? 2 : 1) + 6 * passes) return cudaSuccess;
   *done = true;
   const dim3 grid((unsigned)(triples * C));
   return half ? launch_pdl(hill_sparse_attn_kernel<DT, G, true, kAW / 2>, grid, dim3(kAThreads / 2), AttnCfg::smem(kAW / 2),

@@ -77,6 +77,8 @@ def test_attention_over_every_split(H, case, dtype):
 @pytest.mark.parametrize("B,Hq,Hkv,n,kept,max_k,launches", [
     (8, 32, 32, 4096, [819] * 8, 819, 1), (8, 32, 32, 4096, [819] + [0] * 7, 819, 1),
     (8, 32, 32, 4096, [947, 0, 1, 31, 600, 0, 0, 33], 947, 1),
+    (8, 32, 8, 5000, [4600, 0, 1, 31, 600, 4000, 0, 33], 4600, 1),   # groups: one round more
+    (8, 32, 8, 6000, [5600, 0, 1, 31, 600, 4000, 0, 33], 5600, 2),
     (4, 32, 32, 4096, [3277, 200, 0, 200], 3277, 2),    # one long sequence: its batches over all warps
     (6, 40, 40, 2048, [1500, 50, 50, 0, 50, 1], 1500, 2),
     (1, 32, 32, 4096, [3277], 3277, 1), (2, 32, 32, 4096, [3277, 1], 3277, 1),
